@@ -239,9 +239,11 @@ __device__ __forceinline__ float2 f2mul(float2 a, float2 b) { return __fmul2_rn(
 // their four parts: each is kept as mantissa * 2^e with the pair's e.  The
 // smaller product keeps its full FP32 precision unless it is below 2^-126 of
 // the larger, where its local-energy term is negligible against the larger one.
+// Exponents count up to 126 only: 2^-127 is no normal number, and of an infinity any
+// positive power of two leaves what it is.
 __device__ __forceinline__ void renorm_pair(float2& x, float2& y, int& e) {
   const float mx = fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(y.x), fabsf(y.y)));
-  int ex = ((__float_as_int(mx) >> 23) & 0xff) - 127;
+  int ex = min((__float_as_int(mx) >> 23) & 0xff, 253) - 127;
   if (mx == 0.f) ex = 0;
   const float sc = __int_as_float((127 - ex) << 23);
   x = f2mul(x, make_float2(sc, sc));
@@ -577,12 +579,13 @@ struct WideSmem {
   uint64_t mbar[2];
   int bad;
   // exponents of a pair's running products: E0 + (E1 << 16) in the first plane, or, for
-  // more units than 16 bits can count (wide_exps), a plane each
+  // more units than 16 bits can count (wide_exps), a plane each.  A tile starts at 127 per
+  // renormalisation to come, which takes off its renorm_scale's field.
   int pe[2][4 * NP][256];
 };
 
 // Whether exponents may need more than 16 bits: a renormalisation (16 units, real: 8)
-// adds at most 128 in magnitude.
+// adds at most 127 in magnitude.
 __host__ __device__ inline bool wide_exps(int mp, bool cplx) {
   return mp / (cplx ? kEBK : kEBK / 2) > 255;
 }
@@ -611,8 +614,13 @@ __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
 }
 
-// The exponent field of a float, in place.
-__device__ __forceinline__ uint32_t exp_bits(float v) { return __float_as_uint(v) & 0x7f800000u; }
+// Bits of the power of two that a renormalisation multiplies v by: 2^(127 - E), E the
+// biased exponent, but never below 2^-126 (renorm_pair has the reason).  127 - E comes
+// from the complemented field, so that the limit costs no instruction (one more per
+// product took 2.5 % of a real call's time).
+__device__ __forceinline__ uint32_t renorm_scale(float v) {
+  return (uint32_t)__viaddmax_s32((int)(~__float_as_uint(v) & 0x7f800000u), -(1 << 23), 1 << 23);
+}
 
 // Sum over the 16 lanes of a configuration (nothing to do where it is zero in the
 // whole warp, as the imaginary parts of a real problem are).
@@ -842,8 +850,9 @@ __device__ __forceinline__ void eloc_wide_body(const CUtensorMap* mtab, const El
           for (int q = 0; q < 4; ++q) {
             Px[p][q] = make_float2(1.f, 1.f);
             if constexpr (CPLX) Py[p][q] = make_float2(0.f, 0.f);
-            S.pe[0][p * 4 + q][tid] = 0;
-            if (big) S.pe[1][p * 4 + q][tid] = 0;
+            const int e = 127 * (CPLX ? 1 : 2) * nchunk;
+            S.pe[0][p * 4 + q][tid] = big ? e : e * 65537;
+            if (big) S.pe[1][p * 4 + q][tid] = e;
           }
         }
       }
@@ -860,22 +869,20 @@ __device__ __forceinline__ void eloc_wide_body(const CUtensorMap* mtab, const El
           for (int q = 0; q < 4; ++q) {
             uint32_t b0, b1;
             if constexpr (CPLX) {
-              b0 = exp_bits(fmaxf(fabsf(Px[p][q].x), fabsf(Py[p][q].x)));
-              b1 = exp_bits(fmaxf(fabsf(Px[p][q].y), fabsf(Py[p][q].y)));
+              b0 = renorm_scale(fmaxf(fabsf(Px[p][q].x), fabsf(Py[p][q].x)));
+              b1 = renorm_scale(fmaxf(fabsf(Px[p][q].y), fabsf(Py[p][q].y)));
             } else {
-              b0 = exp_bits(Px[p][q].x);
-              b1 = exp_bits(Px[p][q].y);
+              b0 = renorm_scale(Px[p][q].x);
+              b1 = renorm_scale(Px[p][q].y);
             }
-            // 2^(127 - E), E the biased exponent (zero: any power of two will do)
-            const float2 sc = make_float2(__uint_as_float(0x7f000000u - b0),
-                                          __uint_as_float(0x7f000000u - b1));
+            const float2 sc = make_float2(__uint_as_float(b0), __uint_as_float(b1));
             Px[p][q] = f2mul(Px[p][q], sc);
             if constexpr (CPLX) Py[p][q] = f2mul(Py[p][q], sc);
             if (big) {
-              S.pe[0][p * 4 + q][tid] += (int)(b0 >> 23) - 127;
-              S.pe[1][p * 4 + q][tid] += (int)(b1 >> 23) - 127;
+              S.pe[0][p * 4 + q][tid] -= (int)(b0 >> 23);
+              S.pe[1][p * 4 + q][tid] -= (int)(b1 >> 23);
             } else {
-              S.pe[0][p * 4 + q][tid] += (int)((b0 >> 23) + (b1 >> 23) * 65536u) - 127 * 65537;
+              S.pe[0][p * 4 + q][tid] -= (int)((b0 >> 23) + (b1 >> 7));
             }
           }
       };
