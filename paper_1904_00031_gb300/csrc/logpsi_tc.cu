@@ -1,8 +1,8 @@
 // K1 (tensor-core path): theta = [W | b] [sigma; 1] on the tensor cores (W | b
 // split into BF16 hi + lo planes by nk_rbm_prepare, sigma exact in BF16, FP32
 // accumulation in TMEM), ln cosh fused into the epilogue and summed per
-// configuration in FP64, a . sigma added in FP64 (Sec. 2.2.2, RbmSpin).  With
-// logpsi NULL the epilogue only stores theta and / or tanh(theta).
+// configuration in FP64, a . sigma summed exactly as 64-bit integers (Sec. 2.2.2,
+// RbmSpin).  With logpsi NULL the epilogue only stores theta and / or tanh(theta).
 #include <vector>
 
 #include "tc.cuh"
