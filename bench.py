@@ -763,8 +763,7 @@ def run_gpu_supervised(args):
     flops = 3.0 * ns * (4 if cplx else 2) * n * m
     pk, src = peaks()
     peak = pk.get("bf16_tflops_sustained", pk["bf16_tflops"])
-    chunks = (ns + 16383) // 16384
-    launches = 1 + 3 + chunks * (5 + (1 if chunks > 1 else 0)) + 1 + 1 + 2
+    launches = nk.count_kernels(lambda: step(0))
     achieved = flops / (ms / 1e3) / 1e12
     return rank, {
         "metric": "supervised overlap learning (Eq. 1 loss, gradient, AdaMax) target samples/s",
@@ -864,7 +863,7 @@ def run_gpu_ffnn(args):
     f_fl = float(ns) * sum(per)
     b_fl = float(ns) * (sum(per) + sum(8 * widths[l] * widths[l - 1] for l in range(2, L + 1)))
     ach = (f_fl + b_fl) / (ms / 1e3) / 1e12
-    launches = (L + 1) + 4 * L
+    launches = nk.count_kernels(lambda: step(0))
     big = ns * sum(widths[1:]) * 16 > 129e6
     return rank, {
         "metric": "multi-layer ln cosh FFNN ln psi + gradient, samples/s",

@@ -17,12 +17,13 @@ import torch
 
 from . import nk
 from . import workloads as W
-from .vmc import VmcSr, adj_centres, centring_fused
+from .vmc import VmcSr
 
 
 def _metro_template(w) -> tuple:
-    """The Metropolis kernel template an instance runs: the library's built-in
-    rule, for counting the fused launches.  One CTA per proposal group (complex
+    """The Metropolis kernel template an instance runs by the library's built-in
+    rule (instances are only grouped by it: another rule would give the same
+    results from launches that overlap less).  One CTA per proposal group (complex
     RBMs, group size <= 8, m <= 256 or > 2048): (unit pairs per thread, block
     size); else warps per chain: (field, hidden units per lane, warps per chain,
     group size)."""
@@ -168,34 +169,10 @@ class BatchedVmc:
         return [v.info() for v in self.items]
 
     def launches_per_step(self) -> int:
-        if self.fused:
-            fields = len({v.w.is_complex for v in self.items})
-            # sampling, per kernel template (one call each, on its own stream): the
-            # move rows, the sweep launch, the device counters (graph mode); up to
-            # 64 items per launch
-            n = len(self.sweep_groups) * (2 + (1 if self.use_graph else 0))
-            n += fields            # theta
-            # local energies: real problems of several 64-move tiles and complex ones of
-            # whole tiles run their own (move table, energies; complex: both forms),
-            # the others share a move-table launch and one launch per field
-            real = [v for v in self.items if not v.w.is_complex]
-            cplx = [v for v in self.items if v.w.is_complex]
-            own = sum(v.op.n_moves > 64 for v in real), \
-                sum(v.op.n_moves > 0 and v.op.n_moves % 64 == 0 for v in cplx)
-            shared = (len(real) > own[0]) + (len(cplx) > own[1])
-            n += 2 * own[0] + 3 * own[1] + (1 + shared if shared else 0)
-        elif self.srb is None:
-            return sum(v.launches_per_step() for v in self.items)
-        else:
-            n = sum(v.launches_per_step() - v.sr_launches() for v in self.items)
-        if self.srb is None:
-            return n + sum(v.sr_launches() for v in self.items)
-        groups = (len(self.items) + 63) // 64   # up to 64 instances per launch
-        # per group: statistics (3), flags, sigma' planes (2), force, CG start (2),
-        # 7 per CG iteration (6 when every forward writes its centring partials, 5
-        # when every adjoint also centres its input)
-        # plus the first iteration's planes, update, prepare (2)
-        fused = all(centring_fused(v.ns, v.w.m, v.w.is_complex) for v in self.items)
-        adj = fused and all(adj_centres(v.w.m, v.w.is_complex) for v in self.items)
-        per = 5 if adj else (6 if fused else 7)
-        return n + groups * (3 + 1 + 2 + 2 + 2 + per * self.sr_args[2] + 1 + 3)
+        """Kernel launches of one iteration of all instances, counted as
+        VmcSr.launches_per_step counts them."""
+        counters = [v.chains._s.counter for v in self.items]
+        n = nk.count_kernels(self._eager_step)
+        for v, c in zip(self.items, counters):
+            v.chains._s.counter = c
+        return n

@@ -194,6 +194,29 @@ def _require_gpu(*tensors):
             raise NkError("nk: every tensor argument must live on the CUDA device")
 
 
+def count_kernels(fn) -> int:
+    """Kernel launches of fn(), from the nodes of its capture into a CUDA graph that is
+    thrown away (nothing runs; call after fn() has run once).  Synchronises."""
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g, capture_error_mode="relaxed"):
+        fn()
+    cu, n, kind = C.CDLL("libcuda.so.1"), C.c_size_t(0), C.c_int(0)
+    graph = C.c_void_p(g.raw_cuda_graph())
+
+    def check(err):
+        if err:
+            raise NkError(f"count_kernels: CUDA driver error {err}")
+
+    check(cu.cuGraphGetNodes(graph, None, C.byref(n)))
+    nodes = (C.c_void_p * n.value)()
+    check(cu.cuGraphGetNodes(graph, nodes, C.byref(n)))
+    kernels = 0
+    for node in nodes:
+        check(cu.cuGraphNodeGetType(C.c_void_p(node), C.byref(kind)))
+        kernels += kind.value == 0  # CU_GRAPH_NODE_TYPE_KERNEL
+    return kernels
+
+
 # ---------------------------------------------------------------------- RBM
 
 class Rbm:

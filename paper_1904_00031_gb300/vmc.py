@@ -15,33 +15,11 @@ from . import nk
 from . import workloads as W
 
 
-def centring_fused(ns: int, m: int, is_complex: bool) -> bool:
-    """Whether the tensor-core SR forward writes the centring partials itself:
-    one per CTA (sample tiles x hidden-tile halves) must fit 1024 slots.  The
-    halves rule is the library's: two when the hidden tiles are at least two
-    and twice the CTAs fill their last wave of 152 better."""
-    tiles = (ns + 127) // 128
-    mt = (m + 1 + (63 if is_complex else 127)) // (64 if is_complex else 128)
-
-    def eff(b):
-        return b / (((b + 151) // 152) * 152)
-
-    nseg = 2 if mt >= 2 and eff(2 * tiles) > eff(tiles) else 1
-    return tiles * nseg <= 1024
-
-
 def error_blocks(n_chains: int, group_size: int) -> int:
     """Independent units of the energy error bar: the chains of one proposal
     group share their proposal sequence, so whole groups are the blocks (one
     block, i.e. no error bar, when the chains do not split into whole groups)."""
     return n_chains // group_size if n_chains % group_size == 0 else 1
-
-
-def adj_centres(m: int, is_complex: bool) -> bool:
-    """Whether the SR adjoint centres the forward's output itself (at most four
-    parameter tiles of 64 complex or 128 real hidden units)."""
-    per = 64 if is_complex else 128
-    return (m + 1 + per - 1) // per <= 4
 
 
 class VmcSr:
@@ -170,41 +148,6 @@ class VmcSr:
                 self.w.n_chains * sweeps * (self.replicas - 1) / 2)
         return d
 
-    def sr_launches(self) -> int:
-        """Kernel launches of one SR step: statistics (3), force and CG start, the
-        CG iterations, the update and the refreshed planes (2)."""
-        # per CG iteration: forward, adjoint and the fused vector kernel; the centring
-        # (its partials, its application) where the contractions do not do it
-        # themselves; symmetric steps run the vector kernels unfused (3)
-        vec = 3 if isinstance(self, VmcSrSymm) else 1
-        if self.prec == nk.NK_PREC_BF16X2:
-            fused = centring_fused(self.ns, self.w.m, self.w.is_complex)
-            ctr = (0 if adj_centres(self.w.m, self.w.is_complex) else 1) if fused else 2
-            # sigma'^T, sigma' rows, adjoint, reduction, CG start (2); the first
-            # iteration also builds the planes of p
-            return 3 + 6 + (2 + ctr + vec) * self.w.n_cg + 1 + 3
-        pa = (self.w.n + 1) * (self.w.m + 1)
-        top = 20 if self.ns <= 1536 else 18 if self.w.is_complex else 19
-        if vec == 1 and pa <= 1024 and self.w.m <= 63 and self.ns <= 4096 and self.ns * pa <= 1 << top:
-            return 3 + 4 + 1 + 3  # the whole CG in one launch
-        blocks = (self.ns + 63) // 64 if self.ns < 2 * 152 * 128 else (self.ns + 127) // 128
-        ctr = 2 if blocks > 1024 else (0 if self._fp32_adjoint_centres() else 1)
-        # adjoint, reduction, CG start (2), the first F32 copy of p
-        return 3 + 4 + 1 + (2 + ctr + vec) * self.w.n_cg + 3
-
-    def _fp32_adjoint_centres(self) -> bool:
-        """Whether the FP32 adjoint centres its input itself (the library's rule: at
-        most 16 tiles and 1024 samples per split)."""
-        n1, m1, ns = self.w.n + 1, self.w.m + 1, self.ns
-        cdiv = lambda x, a: (x + a - 1) // a
-        tiles64 = cdiv(n1, 64) * cdiv(m1, 64)
-        splits = max(1, min((2 * 152 + tiles64 - 1) // tiles64, max(1, ns // 256), 64))
-        if self.rbm._s.sr_splits > 0:
-            splits = max(1, min(int(self.rbm._s.sr_splits), cdiv(ns, 64)))
-        chunk = cdiv(cdiv(ns, splits), 16) * 16
-        tiles = cdiv(m1, 64) * cdiv(n1, 64 if self.w.is_complex else 128)
-        return chunk <= 1024 and tiles <= 16
-
     def param_tensors(self):
         """The FP64 master parameters a caller uploads (device tensors)."""
         return [self.rbm.a, self.rbm.b, self.rbm.w]
@@ -215,18 +158,16 @@ class VmcSr:
 
     # kernel launches per step (for reporting)
     def launches_per_step(self) -> int:
-        # move rows, sweep; with tempering a sweep launch and an exchange launch
-        # per sweep (the rows once)
-        n = 2
-        sweeps = self.w.n_discard + self.w.samples_per_chain
-        if self.replicas > 1:
-            n += 2 * sweeps - 1
-        if self.use_graph:  # the device counter is advanced by a kernel after each sweep launch
-            n += sweeps if self.replicas > 1 else 1
-        n += 1                                                  # ln psi / theta
-        n += 2                                                  # move tables, local energy
-        n += self.sr_launches()                                 # SR step
+        """Kernel launches of one iteration, counted in its captured graph (after at
+        least one step; nothing runs, and a host-side proposal counter stays put)."""
+        counter = self.chains._s.counter
+        n = nk.count_kernels(self._eager_step)
+        self.chains._s.counter = counter
         return n
+
+    def sr_launches(self) -> int:
+        """Kernel launches of the iteration's SR step, counted likewise."""
+        return nk.count_kernels(self.sr)
 
 
 class VmcSrSymm(VmcSr):
@@ -254,11 +195,3 @@ class VmcSrSymm(VmcSr):
 
     def refresh(self):
         nk.nk_symm_expand(self.sy)
-
-    def sr_launches(self) -> int:
-        """As the untied step, plus per CG iteration the expansion of p, its planes
-        and the fold of S p (tensor cores; expansion and fold on the FP32 path),
-        the fold of F, and the expansion of the updated parameters."""
-        if self.prec == nk.NK_PREC_BF16X2:
-            return super().sr_launches() + 3 * self.w.n_cg + 1
-        return super().sr_launches() + 3 * self.w.n_cg + 2
