@@ -474,7 +474,8 @@ nk_status nk_tune_shapes(nk_rbm* rbm, const void* op_dev, int32_t n_moves, const
  * (nk_rbm.sampler) equal unit pairs per thread and block size -- one
  * device-counter launch; ln psi:
  * one launch per field; local energies: the move tables of all items, one
- * energy launch per field), each item running the arithmetic of its own call.
+ * energy launch per field, kernel form, tile and cluster size), each item
+ * running the arithmetic of its own call.
  * (With graph capture, the fused launches are single nodes.) */
 typedef struct nk_logpsi_item {
   const nk_rbm* rbm;

@@ -18,6 +18,7 @@
 #include <stddef.h>
 #include <string.h>
 
+#include <memory>
 #include <type_traits>
 
 namespace nk {
@@ -224,7 +225,8 @@ __global__ void move_tables_batch_kernel(const __grid_constant__ MoveTableBatch 
     const OpDevHeader* H = reinterpret_cast<const OpDevHeader*>(J.op);
     const OpMove* mvs = reinterpret_cast<const OpMove*>(J.op + H->off_moves);
     if (J.cplx)
-      move_job_elem<true>(x - B.start[lo], mvs, J.tab, J.a, J.mp, J.nm, J.nm_pad, false, J.out);
+      move_job_elem<true>(x - B.start[lo], mvs, J.tab, J.a, J.mp, J.nm, J.nm_pad,
+                          (H->flags & kOpQuadMoves) != 0, J.out);
     else
       move_job_elem<false>(x - B.start[lo], mvs, J.tab, J.a, J.mp, J.nm, J.nm_pad, false, J.out);
   }
@@ -1125,13 +1127,15 @@ __global__ void __launch_bounds__(256, 2) local_energy_batch(const __grid_consta
   local_energy_body(&B.map[k], A, b / A.nseg, b % A.nseg);
 }
 
-template <int NP>
+// (CLUSTER: every problem's tiles are shared by `parts` CTAs, so that the problems start
+// at whole clusters)
+template <bool CPLX, int NP, bool CLUSTER>
 __global__ void __launch_bounds__(256, 2)
-    local_energy_wide_batch(const __grid_constant__ ElocBatch B) {
+    local_energy_wide_batch(const __grid_constant__ ElocBatch B, int parts) {
   int k = 0;
   while (k + 1 < B.n && (int)blockIdx.x >= B.start[k + 1]) ++k;
-  eloc_wide_body<false, NP, false>(&B.map[k], B.a[k], (int)blockIdx.x - B.start[k],
-                                   B.start[k + 1] - B.start[k], 1);
+  eloc_wide_body<CPLX, NP, CLUSTER>(&B.map[k], B.a[k], (int)blockIdx.x - B.start[k],
+                                    B.start[k + 1] - B.start[k], parts);
 }
 
 size_t local_energy_scratch_bytes(int m, int cplx, int n_moves) {
@@ -1147,7 +1151,9 @@ struct ElocPlan {
   bool cplx;
   size_t smem;
   int64_t blocks;  // configuration tiles of 64 (local_energy_body)
-  bool own;        // in a batch: a call of its own
+  bool wide;       // the wide form may run: real, or whole move tiles of a complex operator
+                   // that may be in the site-quad layout (only the device knows)
+  WidePlan wp;
   MoveTableJob job;
   int64_t tab_elems;
 };
@@ -1201,9 +1207,14 @@ static nk_status plan_local_energy(const nk_rbm* r, const void* op_dev, int n_mo
   A.nseg = (ntile >= 2 && wave_eff(2 * P->blocks) > wave_eff(P->blocks)) ? 2 : 1;
   if (r->eloc_segs > 0) A.nseg = (r->eloc_segs >= 2 && ntile >= 2) ? 2 : 1;  // tuned or set
   A.seg_fast = A.nseg == 2 && P->blocks <= 65535 ? 1 : 0;
-  // (several move tiles of a real problem are summed as its size has it, wide_plan)
-  P->own = cplx ? n_moves > 0 && n_moves % kEBM == 0 : ntile >= 2;
+  P->wide = !cplx || (n_moves > 0 && n_moves % kEBM == 0);
+  if (P->wide) P->wp = wide_plan(ns, n_moves, cplx);
   return NK_OK;
+}
+
+// Whether CTAs of one form or the other add their sums up in eloc, which starts at zero.
+static bool adds_up(const ElocPlan& P) {
+  return (P.cplx && P.A.nseg == 2) || (P.wide && P.wp.ranges);
 }
 
 nk_status launch_local_energy(const nk_rbm* r, const void* op_dev, int n_moves,
@@ -1224,12 +1235,8 @@ nk_status launch_local_energy(const nk_rbm* r, const void* op_dev, int n_moves,
                                                                   n_moves, P.job.nm_pad, scratch);
     if (nk_status e = check_launch("nk_local_energy(move tables)")) return e;
   }
-  // a complex operator may be in the site-quad layout (only the device knows) if it has
-  // whole tiles of 64 moves
-  const bool wide = !P.cplx || P.own;
-  const WidePlan wp = wide_plan(ns, n_moves, P.cplx);
-  if ((P.cplx && A.nseg == 2 || wide && wp.ranges) &&
-      cudaMemsetAsync(eloc, 0, (size_t)ns * 2 * sizeof(double), st) != cudaSuccess)
+  const WidePlan& wp = P.wp;
+  if (adds_up(P) && cudaMemsetAsync(eloc, 0, (size_t)ns * 2 * sizeof(double), st) != cudaSuccess)
     return fail(NK_ERR_CUDA, "nk_local_energy: cudaMemsetAsync failed");
   auto set_smem = [](auto kern, size_t smem) {
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ==
@@ -1253,7 +1260,7 @@ nk_status launch_local_energy(const nk_rbm* r, const void* op_dev, int n_moves,
       return fail(NK_ERR_CUDA, "nk_local_energy: launch failed");
     return NK_OK;
   };
-  if (wide) {
+  if (P.wide) {
     // complex: only the device knows the operator's layout, and the kernel that it is
     // not for returns
     // one CTA per tile: ranges of whole tiles
@@ -1278,10 +1285,94 @@ nk_status launch_local_energy(const nk_rbm* r, const void* op_dev, int n_moves,
   return check_launch("nk_local_energy");
 }
 
-// Fused local energies of many problems: one move-table launch for all of them,
-// one launch of the energy kernel per field (at most kElocBatch problems each).
-// Every problem runs its own launch's arithmetic and move-tile split, so the
-// results are those of separate calls.
+// Problems that a launch of the batch takes, started one after another.
+static void batch_add(ElocBatch* B, const ElocPlan& P, int64_t ctas) {
+  B->a[B->n] = P.A;
+  B->map[B->n] = P.map;
+  B->start[B->n + 1] = B->start[B->n] + (int)ctas;
+  ++B->n;
+}
+
+// The wide form of a batch's problems, one launch per field, tile and cluster size (at
+// most kElocBatch problems each).  A problem keeps the cluster size and ranges of its own
+// call, which fix the order of its sums; where one CTA takes a whole tile the sums do not
+// depend on the tile, and 64 configurations are taken where 128 leave SMs idle.
+static nk_status launch_wide_batch(const std::vector<ElocPlan>& plans, cudaStream_t st) {
+  const int n = (int)plans.size();
+  int64_t c64[2] = {0, 0};  // tiles of 64 of the problems that are free to choose
+  auto free_np = [&](const ElocPlan& P) { return P.wp.parts == 1 && !P.wp.ranges; };
+  for (const ElocPlan& P : plans)
+    if (P.wide && free_np(P)) c64[P.cplx] += (P.A.ns + 63) / 64;
+  auto np_of = [&](const ElocPlan& P) {
+    return free_np(P) ? (c64[P.cplx] <= 2 * 152 ? 2 : 4) : P.wp.np;
+  };
+  std::vector<bool> done((size_t)n, false);
+  std::unique_ptr<ElocBatch> B(new ElocBatch);  // 15 KB: kept off the stack
+  for (int u = 0; u < n; ++u) {
+    if (done[u] || !plans[u].wide) continue;
+    const bool cplx = plans[u].cplx;
+    const int np = np_of(plans[u]);
+    int parts = plans[u].wp.parts;
+    size_t smem = 0;
+    B->n = 0;
+    B->start[0] = 0;
+    for (int v = u; v < n && B->n < kElocBatch; ++v) {
+      const ElocPlan& P = plans[v];
+      if (done[v] || !P.wide || P.cplx != cplx || np_of(P) != np || P.wp.parts != parts) continue;
+      done[v] = true;
+      batch_add(B.get(), P, free_np(P) ? (P.A.ns + 32 * np - 1) / (32 * np) : P.wp.grid);
+      smem = std::max(smem, cplx ? (np == 4 ? wide_smem<true, 4>(P.A.mp) : wide_smem<true, 2>(P.A.mp))
+                                 : (np == 4 ? wide_smem<false, 4>(P.A.mp) : wide_smem<false, 2>(P.A.mp)));
+    }
+    const int64_t ctas = B->start[B->n];
+    auto go = [&](auto kern, int64_t alone) -> nk_status {
+      // few clusters: one CTA per SM (kAloneSmem)
+      if (ctas / parts <= alone) smem = std::max(smem, kAloneSmem);
+      if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+          cudaSuccess)
+        return fail(NK_ERR_CUDA, "nk_batch_local_energy: shared memory attribute");
+      cudaLaunchConfig_t cfg{};
+      cfg.gridDim = dim3((unsigned)ctas);
+      cfg.blockDim = dim3(256);
+      cfg.dynamicSmemBytes = smem;
+      cfg.stream = st;
+      cudaLaunchAttribute at{};
+      at.id = cudaLaunchAttributeClusterDimension;
+      at.val.clusterDim.x = (unsigned)parts;
+      at.val.clusterDim.y = at.val.clusterDim.z = 1;
+      cfg.attrs = &at;
+      cfg.numAttrs = parts > 1 ? 1 : 0;
+      void* args[] = {B.get(), &parts};
+      if (cudaLaunchKernelExC(&cfg, (const void*)kern, args) != cudaSuccess)
+        return fail(NK_ERR_CUDA, "nk_batch_local_energy: launch failed");
+      return NK_OK;
+    };
+    auto pick = [&](auto r4, auto r2, auto c4, auto c2, int64_t alone) {
+      if (parts > 1) return np == 4 ? go(c4, alone) : go(c2, alone);
+      return np == 4 ? go(r4, 0) : go(r2, 0);
+    };
+    const nk_status e =
+        cplx ? pick(local_energy_wide_batch<true, 4, false>, local_energy_wide_batch<true, 2, false>,
+                    local_energy_wide_batch<true, 4, true>, local_energy_wide_batch<true, 2, true>,
+                    parts > 1 ? (np == 4 ? wide_clusters<true, 4>(parts, true)
+                                         : wide_clusters<true, 2>(parts, true)) : 0)
+             : pick(local_energy_wide_batch<false, 4, false>, local_energy_wide_batch<false, 2, false>,
+                    local_energy_wide_batch<false, 4, true>, local_energy_wide_batch<false, 2, true>,
+                    parts > 1 ? (np == 4 ? wide_clusters<false, 4>(parts, true)
+                                         : wide_clusters<false, 2>(parts, true)) : 0);
+    if (e) return e;
+  }
+  return NK_OK;
+}
+
+// Fused local energies of many problems: one move-table launch for all of them, then
+// one launch of the 4 x 4 form for the complex ones and of the wide form per field, tile
+// and cluster size; of whole move tiles in complex problems, as in single calls, the form
+// that the operator's layout is not for returns at once.  (Problems of several move tiles
+// launched one after another: 48 of 72-site Ising, 256 samples each, 2140 us, here 119;
+// 48 of 64-site Heisenberg, 1024 samples each, 2535, here 201.)
+// Every problem runs its own launch's arithmetic and move-tile split, so the results are
+// those of separate calls.
 nk_status launch_local_energy_fused(const nk_eloc_item* items, const int* idx, int n,
                                     cudaStream_t st) {
   std::vector<ElocPlan> plans((size_t)n);
@@ -1291,17 +1382,6 @@ nk_status launch_local_energy_fused(const nk_eloc_item* items, const int* idx, i
                                         it.eloc_out, it.t_out, it.scratch, it.scratch_bytes,
                                         &plans[u]))
       return e;
-  }
-  // complex problems that may have a site-quad operator, real ones of several move tiles:
-  // calls of their own
-  for (int u = 0; u < n; ++u) {
-    if (!plans[u].own) continue;
-    const nk_eloc_item& it = items[idx[u]];
-    if (nk_status e = launch_local_energy(it.rbm, it.op_dev, it.n_moves, it.sigma, it.theta, it.ns,
-                                          it.eloc_out, it.t_out, it.scratch, it.scratch_bytes, st))
-      return e;
-    plans[u].blocks = plans[u].tab_elems = 0;  // done
-    plans[u].A.nseg = 1;
   }
   for (int u0 = 0; u0 < n; u0 += kMoveJobs) {
     MoveTableBatch TB;
@@ -1320,52 +1400,27 @@ nk_status launch_local_energy_fused(const nk_eloc_item* items, const int* idx, i
       if (nk_status e = check_launch("nk_batch_local_energy(move tables)")) return e;
     }
   }
-  for (int u = 0; u < n; ++u)
-    if (plans[u].A.nseg == 2 &&
-        cudaMemsetAsync(plans[u].A.eloc, 0, (size_t)plans[u].A.ns * 2 * sizeof(double), st) !=
-            cudaSuccess)
+  for (const ElocPlan& P : plans)
+    if (adds_up(P) &&
+        cudaMemsetAsync(P.A.eloc, 0, (size_t)P.A.ns * 2 * sizeof(double), st) != cudaSuccess)
       return fail(NK_ERR_CUDA, "nk_batch_local_energy: cudaMemsetAsync failed");
-  for (int field = 0; field < 2; ++field) {
-    const bool cplx = field == 1;
-    for (int u0 = 0; u0 < n;) {
-      ElocBatch* B = new ElocBatch;  // about 11 KB: kept off the stack
-      B->n = 0;
-      B->start[0] = 0;
-      size_t smem = 0;
-      // 64-configuration tiles of the wide form where they leave SMs idle
-      int64_t c64 = 0;
-      for (int v = u0; v < n; ++v)
-        if (!plans[v].cplx && plans[v].blocks > 0) c64 += (plans[v].A.ns + 63) / 64;
-      const int np = c64 <= 2 * 152 ? 2 : 4;
-      int u = u0;
-      for (; u < n && B->n < kElocBatch; ++u) {
-        const ElocPlan& P = plans[u];
-        if (P.cplx != cplx || P.blocks == 0) continue;
-        B->a[B->n] = P.A;
-        B->map[B->n] = P.map;
-        B->start[B->n + 1] = B->start[B->n] + (int)(cplx ? P.blocks * P.A.nseg : (P.A.ns + 32 * np - 1) / (32 * np));
-        ++B->n;
-        smem = std::max(smem, cplx      ? P.smem
-                              : np == 4 ? wide_smem<false, 4>(P.A.mp)
-                                        : wide_smem<false, 2>(P.A.mp));
-      }
-      u0 = u;
-      nk_status e = NK_OK;
-      if (B->n > 0) {
-        auto kern = cplx      ? local_energy_batch
-                    : np == 4 ? local_energy_wide_batch<4>
-                              : local_energy_wide_batch<2>;
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-            cudaSuccess)
-          e = fail(NK_ERR_CUDA, "nk_batch_local_energy: shared memory attribute");
-        else {
-          kern<<<(unsigned)B->start[B->n], 256, smem, st>>>(*B);
-          e = check_launch("nk_batch_local_energy");
-        }
-      }
-      delete B;
-      if (e) return e;
+  if (nk_status e = launch_wide_batch(plans, st)) return e;
+  std::unique_ptr<ElocBatch> B(new ElocBatch);
+  for (int u = 0; u < n;) {
+    size_t smem = 0;
+    B->n = 0;
+    B->start[0] = 0;
+    for (; u < n && B->n < kElocBatch; ++u) {
+      if (!plans[u].cplx) continue;
+      batch_add(B.get(), plans[u], plans[u].blocks * plans[u].A.nseg);
+      smem = std::max(smem, plans[u].smem);
     }
+    if (B->n == 0) continue;
+    if (cudaFuncSetAttribute(local_energy_batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)smem) != cudaSuccess)
+      return fail(NK_ERR_CUDA, "nk_batch_local_energy: shared memory attribute");
+    local_energy_batch<<<(unsigned)B->start[B->n], 256, smem, st>>>(*B);
+    if (nk_status e = check_launch("nk_batch_local_energy")) return e;
   }
   return NK_OK;
 }
