@@ -256,8 +256,14 @@ constexpr bool metro_may_reside() {
   return NU <= (CPLX ? 4 : 16);
 }
 
-// Two CTAs of 512 threads (four of 256) per SM where a thread's units fit 64 registers.
-#define METRO_BOUNDS(CPLX, NU) __launch_bounds__(512, ((CPLX) ? (NU) <= 4 : (NU) <= 16) ? 2 : 1)
+// CTAs of 512 threads per SM that a template can be compiled for: two (four of 256) where
+// a thread's units fit 64 registers.  A launch whose CTAs all fit at 128 registers takes
+// them: 96 x 384 real, 1024 chains 356 us at 64 registers, 252 at 128; 400 x 512 (two
+// warps per chain) 1499 and 1246; but 16,384 chains 1739 and 1939, 14,065 and 17,137.
+template <bool CPLX, int NU>
+constexpr int metro_max_ctas() {
+  return NU <= (CPLX ? 4 : 16) ? 2 : 1;
+}
 
 // The instantiated NU of (field, warps per chain) below NU: a problem that runs with NU
 // needs more units per thread than that, so its first units need no bounds check.
@@ -701,8 +707,8 @@ __device__ __forceinline__ void metropolis_body(const MetroArgs& A, const int bx
   }
 }
 
-template <bool CPLX, int NU, int WPC>
-__global__ void METRO_BOUNDS(CPLX, NU) metropolis_kernel(MetroArgs A) {
+template <bool CPLX, int NU, int WPC, int CTAS>
+__global__ void __launch_bounds__(512, CTAS) metropolis_kernel(MetroArgs A) {
   metropolis_body<CPLX, NU, WPC>(A, blockIdx.x);
 }
 
@@ -716,8 +722,9 @@ struct MetroBatch {
   MetroArgs a[kMetroBatch];
 };
 
-template <bool CPLX, int NU, int WPC>
-__global__ void METRO_BOUNDS(CPLX, NU) metropolis_batch_kernel(const __grid_constant__ MetroBatch B) {
+template <bool CPLX, int NU, int WPC, int CTAS>
+__global__ void __launch_bounds__(512, CTAS)
+    metropolis_batch_kernel(const __grid_constant__ MetroBatch B) {
   int k = 0;
   while (k + 1 < B.n && (int)blockIdx.x >= B.start[k + 1]) ++k;
   metropolis_body<CPLX, NU, WPC>(B.a[k], (int)blockIdx.x - B.start[k]);
@@ -913,6 +920,9 @@ size_t metropolis_scratch_bytes(int n, int m, int cplx, int move, int nb) {
   return std::max(bytes, (size_t)round_up((int64_t)rows * (int64_t)grow, 256));
 }
 
+// CTAs that fit the GPU at 128 registers per thread.
+static int metro_roomy(int threads) { return 152 * (512 / threads); }
+
 // Launch functors for the kernel templates: one problem, or a batch of problems
 // sharing a template (field, hidden units per lane, warps per chain, group size).
 struct SingleLaunch {
@@ -921,12 +931,13 @@ struct SingleLaunch {
   cudaStream_t st;
   template <bool CPLX, int NU, int WPC>
   nk_status go() const {
-    auto kern = metropolis_kernel<CPLX, NU, WPC>;
+    const int blocks = (A.nc + A.G - 1) / A.G, threads = 32 * A.G * WPC;
+    auto kern = metropolis_kernel<CPLX, NU, WPC, 1>;
+    if (blocks > metro_roomy(threads)) kern = metropolis_kernel<CPLX, NU, WPC, metro_max_ctas<CPLX, NU>()>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
         cudaSuccess)
       return fail(NK_ERR_CUDA, "nk_metropolis_sweep: cannot reserve %zu B shared memory", smem);
-    const int blocks = (A.nc + A.G - 1) / A.G;
-    kern<<<blocks, 32 * A.G * WPC, smem, st>>>(A);
+    kern<<<blocks, threads, smem, st>>>(A);
     return check_launch("nk_metropolis_sweep");
   }
 };
@@ -938,11 +949,14 @@ struct BatchLaunch {
   cudaStream_t st;
   template <bool CPLX, int NU, int WPC>
   nk_status go() const {
-    auto kern = metropolis_batch_kernel<CPLX, NU, WPC>;
+    const int blocks = B.start[B.n], threads = 32 * G * WPC;
+    auto kern = metropolis_batch_kernel<CPLX, NU, WPC, 1>;
+    if (blocks > metro_roomy(threads))
+      kern = metropolis_batch_kernel<CPLX, NU, WPC, metro_max_ctas<CPLX, NU>()>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
         cudaSuccess)
       return fail(NK_ERR_CUDA, "nk_batch_sweep: cannot reserve %zu B shared memory", smem);
-    kern<<<B.start[B.n], 32 * G * WPC, smem, st>>>(B);
+    kern<<<blocks, threads, smem, st>>>(B);
     return check_launch("nk_batch_sweep");
   }
 };
