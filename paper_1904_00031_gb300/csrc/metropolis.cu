@@ -1068,6 +1068,9 @@ struct MetroPlan {
   int64_t tab_elems;
   uint64_t* ctr_dev;
   uint64_t advance;
+  // all rows resident instead of the ring: their count (0: never) and shared memory
+  int res_rows = 0;
+  size_t res_smem = 0;
 };
 
 static nk_status plan_metropolis(const nk_rbm* r, const nk_chains* ch, int move,
@@ -1194,21 +1197,17 @@ static nk_status plan_metropolis(const nk_rbm* r, const nk_chains* ch, int move,
   const size_t rest = (size_t)round_up(2 * A.G * wpc, 2) * 4 + 2 * kMaxRing * 8 + 16 +
                       (size_t)A.G * wpc * round_up(r->n, 16);
   const size_t cap = 227 * 1024;
-  int ring = rest + 2 * slot > cap ? 0 : (int)std::min<size_t>(kMaxRing, (cap - rest) / slot);
+  const int ring = rest + 2 * slot > cap ? 0 : (int)std::min<size_t>(kMaxRing, (cap - rest) / slot);
   if (ring < 2)
     return fail(NK_ERR_SHAPE,
                 "nk_metropolis_sweep: group_size %d with padded m %d leaves room for fewer "
                 "than two table slots in 227 KB of shared memory",
                 A.G, L.mp);
-  // all rows resident, no ring, where they are small: always up to 32 KB, and up to the
-  // whole shared memory when no second CTA waits for it (at most one per SM).  A step
-  // then waits for no copy and releases no slot (10-site chain, 16 chains: 573 us with
-  // the ring, 385 without).
   const size_t all = (size_t)(move == NK_MOVE_FLIP ? r->n : nb) * slot;
-  A.rows = 0;
-  if (nu <= (cplx ? 4 : 16) && all > 0 && all + rest <= cap &&
-      (all <= 32 * 1024 || (ch->nc + A.G - 1) / A.G <= 152))
-    A.rows = ring = move == NK_MOVE_FLIP ? r->n : nb;
+  if (nu <= (cplx ? 4 : 16) && all > 0 && all + rest <= cap) {
+    P->res_rows = move == NK_MOVE_FLIP ? r->n : nb;
+    P->res_smem = all + rest;
+  }
   A.ring = ring;
   if ((int64_t)(n_discard + n_samples) * r->n > 0x7fffffff)
     return fail(NK_ERR_SHAPE, "nk_metropolis_sweep: too many proposals in one call");
@@ -1240,6 +1239,22 @@ static nk_status plan_metropolis(const nk_rbm* r, const nk_chains* ch, int move,
   return NK_OK;
 }
 
+// All rows resident, no ring: a step then waits for no copy and releases no slot (10-site
+// chain, 16 chains: 573 us with the ring, 385 without).  That pays where every CTA of the
+// call (`ctas`) is on the GPU at once, and beyond while shared memory leaves three
+// quarters of the CTAs that the registers would; 16 problems of 1024 chains, by sites x
+// units and CTAs per SM of four, resident and with the ring: 48 x 96, four, 363 and 474
+// us; 24 x 256, three, 319 and 347; 64 x 128, two, 695 and 670; 16 x 400, two, 443 and
+// 348; 100 x 100, one, 1809 and 1032.
+static void choose_rows(MetroPlan* P, int64_t ctas) {
+  if (P->res_rows == 0) return;
+  const int64_t by_regs = 1024 / (32 * P->A.G * P->wpc);
+  const int64_t per_sm = std::min<int64_t>(228 * 1024 / (P->res_smem + 1024), by_regs);
+  if (ctas > 152 * per_sm && 4 * per_sm < 3 * by_regs) return;
+  P->A.rows = P->A.ring = P->res_rows;
+  P->smem = P->res_smem;
+}
+
 nk_status launch_metropolis(const nk_rbm* r, nk_chains* ch, int move, const int32_t* bi,
                             const int32_t* bk, int nb, int n_discard, int n_samples,
                             int8_t* samples, uint64_t* n_acc, void* scratch, size_t scratch_bytes,
@@ -1249,6 +1264,7 @@ nk_status launch_metropolis(const nk_rbm* r, nk_chains* ch, int move, const int3
                                     n_acc, scratch, scratch_bytes, pt, &P))
     return e;
   if (dry) return NK_OK;  // every check passed; nothing is enqueued
+  choose_rows(&P, (P.A.nc + P.A.G - 1) / P.A.G);
   if (P.tj.kind != kTabNone && P.tab_elems > 0) {
     TableBatch TB;
     TB.n = 1;
@@ -1291,6 +1307,9 @@ nk_status launch_metropolis_fused(const nk_sweep_item* items, const int* idx, in
                                       it.scratch_bytes, nullptr, &plans[u]))
       return e;
   }
+  int64_t ctas = 0;
+  for (const MetroPlan& P : plans) ctas += (P.A.nc + P.A.G - 1) / P.A.G;
+  for (MetroPlan& P : plans) choose_rows(&P, ctas);
   // table builds
   for (int u0 = 0; u0 < n; u0 += kMetroBatch) {
     TableBatch TB;

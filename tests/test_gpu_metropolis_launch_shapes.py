@@ -70,3 +70,19 @@ def test_batch_registers_per_thread(nk, chains):
     nk.nk_batch_sweep([j for j, *_ in probs])
     for j, *ref in probs:
         check(j, *ref)
+
+
+# The rows' bytes leave room for three CTAs per SM (of eight by registers), one (of four), two,
+# three (which is enough beyond what fits at once, too).
+@pytest.mark.parametrize("move,n,m,cplx,G,fit", [("flip", 24, 256, False, 4, 3),
+                                                 ("flip", 96, 192, False, 8, 1),
+                                                 ("exchange", 130, 32, True, 8, 2),
+                                                 ("flip", 24, 256, False, 8, 3)])
+@pytest.mark.parametrize("over", [0, 1])
+def test_batch_rows(nk, move, n, m, cplx, G, fit, over):
+    """As many CTAs in a call as fit with their rows resident, and one more."""
+    ctas = 152 * fit + over
+    probs = [problem(nk, move, n, m, cplx, G, k * G) for k in (40, ctas - 90, 50)]
+    nk.nk_batch_sweep([j for j, *_ in probs])
+    for j, *ref in probs:
+        check(j, *ref)
