@@ -17,6 +17,18 @@ nk_status fail(nk_status s, const char* fmt, ...);
 // NK_ERR_CUDA with the pending launch error, or NK_OK.
 nk_status check_launch(const char* where);
 
+// Lets a kernel take `smem` bytes of dynamic shared memory.  The limit is one per kernel
+// whatever thread or stream launches it, so it is always set to the same value, the most
+// that the kernel may ask for (an SM gives 227 KB, less the kernel's static shared memory:
+// at most 1 KB): set to each call's own need, it made a larger call's launch in another
+// thread fail.
+template <class K>
+bool allow_smem(K* kern, size_t smem, size_t most = 226 * 1024) {
+  return smem <= most && cudaFuncSetAttribute((const void*)kern,
+                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)most) == cudaSuccess;
+}
+
 nk_status launch_prepare(const nk_rbm* r, cudaStream_t st);
 
 // Device status words (status.cuh): OR each translation unit's word into *out

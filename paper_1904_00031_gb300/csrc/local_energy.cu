@@ -1038,8 +1038,7 @@ static int64_t wide_slots(K kern, size_t smem, int parts) {
   cfg.attrs = &at;
   cfg.numAttrs = 1;
   int n = 0;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-          cudaSuccess ||
+  if (!allow_smem(kern, smem) ||
       cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) {
     cudaGetLastError();
     return 1;
@@ -1238,13 +1237,9 @@ nk_status launch_local_energy(const nk_rbm* r, const void* op_dev, int n_moves,
   const WidePlan& wp = P.wp;
   if (adds_up(P) && cudaMemsetAsync(eloc, 0, (size_t)ns * 2 * sizeof(double), st) != cudaSuccess)
     return fail(NK_ERR_CUDA, "nk_local_energy: cudaMemsetAsync failed");
-  auto set_smem = [](auto kern, size_t smem) {
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ==
-           cudaSuccess;
-  };
   auto go_wide = [&](auto kern, size_t smem) -> nk_status {
     if (wp.alone && wp.parts > 1) smem = std::max(smem, kAloneSmem);
-    if (!set_smem(kern, smem)) return fail(NK_ERR_CUDA, "nk_local_energy: shared memory attribute");
+    if (!allow_smem(kern, smem)) return fail(NK_ERR_CUDA, "nk_local_energy: shared memory attribute");
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)wp.grid);
     cfg.blockDim = dim3(256);
@@ -1277,7 +1272,7 @@ nk_status launch_local_energy(const nk_rbm* r, const void* op_dev, int n_moves,
                       local_energy_wide<false, 4, true>, local_energy_wide<false, 2, true>);
     if (e || !P.cplx) return e;
   }
-  if (!set_smem(local_energy_tiled, P.smem))
+  if (!allow_smem(local_energy_tiled, P.smem))
     return fail(NK_ERR_CUDA, "nk_local_energy: shared memory attribute");
   local_energy_tiled<<<A.seg_fast ? dim3((unsigned)A.nseg, (unsigned)P.blocks)
                                   : dim3((unsigned)P.blocks, (unsigned)A.nseg),
@@ -1328,8 +1323,7 @@ static nk_status launch_wide_batch(const std::vector<ElocPlan>& plans, cudaStrea
     auto go = [&](auto kern, int64_t alone) -> nk_status {
       // few clusters: one CTA per SM (kAloneSmem)
       if (ctas / parts <= alone) smem = std::max(smem, kAloneSmem);
-      if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-          cudaSuccess)
+      if (!allow_smem(kern, smem))
         return fail(NK_ERR_CUDA, "nk_batch_local_energy: shared memory attribute");
       cudaLaunchConfig_t cfg{};
       cfg.gridDim = dim3((unsigned)ctas);
@@ -1416,8 +1410,7 @@ nk_status launch_local_energy_fused(const nk_eloc_item* items, const int* idx, i
       smem = std::max(smem, plans[u].smem);
     }
     if (B->n == 0) continue;
-    if (cudaFuncSetAttribute(local_energy_batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem) != cudaSuccess)
+    if (!allow_smem(local_energy_batch, smem))
       return fail(NK_ERR_CUDA, "nk_batch_local_energy: shared memory attribute");
     local_energy_batch<<<(unsigned)B->start[B->n], 256, smem, st>>>(*B);
     if (nk_status e = check_launch("nk_batch_local_energy")) return e;

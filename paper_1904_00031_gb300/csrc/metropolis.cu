@@ -112,6 +112,8 @@ __device__ __forceinline__ int move_row(const MetroArgs& A, uint64_t ctr, uint32
 // memory (per-thread TMEM columns, loaded and stored with tcgen05.ld /
 // tcgen05.st), which leaves shared memory to the ring.
 constexpr int kMaxRing = 8;
+// a CTA's shared memory at most (all of it dynamic)
+constexpr size_t kMetroSmem = 227 * 1024;
 
 // Complex tables: a thread (half h, lane l) owns units j = 32 (h + WPC q) + l,
 // q < NU, taken in pairs (2 qp, 2 qp + 1).  A row holds one 1024-byte block per
@@ -934,8 +936,7 @@ struct SingleLaunch {
     const int blocks = (A.nc + A.G - 1) / A.G, threads = 32 * A.G * WPC;
     auto kern = metropolis_kernel<CPLX, NU, WPC, 1>;
     if (blocks > metro_roomy(threads)) kern = metropolis_kernel<CPLX, NU, WPC, metro_max_ctas<CPLX, NU>()>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
+    if (!allow_smem(kern, smem, kMetroSmem))
       return fail(NK_ERR_CUDA, "nk_metropolis_sweep: cannot reserve %zu B shared memory", smem);
     kern<<<blocks, threads, smem, st>>>(A);
     return check_launch("nk_metropolis_sweep");
@@ -953,8 +954,7 @@ struct BatchLaunch {
     auto kern = metropolis_batch_kernel<CPLX, NU, WPC, 1>;
     if (blocks > metro_roomy(threads))
       kern = metropolis_batch_kernel<CPLX, NU, WPC, metro_max_ctas<CPLX, NU>()>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
+    if (!allow_smem(kern, smem, kMetroSmem))
       return fail(NK_ERR_CUDA, "nk_batch_sweep: cannot reserve %zu B shared memory", smem);
     kern<<<blocks, threads, smem, st>>>(B);
     return check_launch("nk_batch_sweep");
@@ -969,8 +969,7 @@ struct GroupSingleLaunch {
   template <int PP>
   nk_status go() const {
     auto kern = metropolis_group_kernel<PP>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
+    if (!allow_smem(kern, smem, kMetroSmem))
       return fail(NK_ERR_CUDA, "nk_metropolis_sweep: cannot reserve %zu B shared memory", smem);
     const int blocks = (A.nc + A.G - 1) / A.G;
     kern<<<blocks, threads, smem, st>>>(A);
@@ -986,8 +985,7 @@ struct GroupBatchLaunch {
   template <int PP>
   nk_status go() const {
     auto kern = metropolis_group_batch_kernel<PP>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
+    if (!allow_smem(kern, smem, kMetroSmem))
       return fail(NK_ERR_CUDA, "nk_batch_sweep: cannot reserve %zu B shared memory", smem);
     kern<<<B.start[B.n], threads, smem, st>>>(B);
     return check_launch("nk_batch_sweep");
@@ -1142,7 +1140,7 @@ static nk_status plan_metropolis(const nk_rbm* r, const nk_chains* ch, int move,
     // ring depth: as many row slots as fit next to the partials, barriers and
     // the per-warp spin bytes (theta lives in tensor memory)
     const size_t rest = (size_t)64 * NW + 8 * kMaxRing + 16 + (size_t)NW * round_up(r->n, 16);
-    const size_t cap = 227 * 1024;
+    const size_t cap = kMetroSmem;
     const int ring =
         rest + 2 * row > cap ? 0 : (int)std::min<size_t>(kMaxRing, (cap - rest) / row);
     if (ring < 2)
@@ -1196,7 +1194,7 @@ static nk_status plan_metropolis(const nk_rbm* r, const nk_chains* ch, int move,
   const size_t slot = cd_row + (size_t)L.mp * f + kRowHdr;
   const size_t rest = (size_t)round_up(2 * A.G * wpc, 2) * 4 + 2 * kMaxRing * 8 + 16 +
                       (size_t)A.G * wpc * round_up(r->n, 16);
-  const size_t cap = 227 * 1024;
+  const size_t cap = kMetroSmem;
   const int ring = rest + 2 * slot > cap ? 0 : (int)std::min<size_t>(kMaxRing, (cap - rest) / slot);
   if (ring < 2)
     return fail(NK_ERR_SHAPE,

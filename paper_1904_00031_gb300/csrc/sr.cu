@@ -1515,8 +1515,7 @@ static nk_status launch_cg_small(const CgSmall& A, cudaStream_t st) {
   const size_t f = CPLX ? 8 : 4;
   const size_t smem = sizeof(CgSmallSmem<CPLX>) +
                       f * ((size_t)A.ns + (size_t)ceil_div(A.pa, kCgCtas) * A.splits);
-  if (cudaFuncSetAttribute(cg_small_kernel<CPLX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem) != cudaSuccess)
+  if (!allow_smem(cg_small_kernel<CPLX>, smem))
     return fail(NK_ERR_CUDA, "nk_sr_step: shared memory attribute");
   cg_small_kernel<CPLX><<<kCgCtas, kVecThreads, smem, st>>>(A);
   return check_launch("nk_sr_step(small cg)");

@@ -859,8 +859,7 @@ nk_status launch_fwd_tc(const FwdTcArgs& A, const void* planes, cudaStream_t st)
   }
   const dim3 grid((unsigned)blocks, (unsigned)B.nseg);
   auto go = [&](auto kern, int threads, size_t smem) -> nk_status {
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
+    if (!allow_smem(kern, smem))
       return fail(NK_ERR_CUDA, "fwd_tc: shared memory attribute");
     kern<<<grid, threads, smem, st>>>(map, smap, B);
     return check_launch("fwd_tc");
@@ -933,8 +932,7 @@ nk_status launch_fwd_tc_fused(const FwdTcArgs* args, const void* const* planes, 
       u0 = u;
       if (!e && B->n > 0) {
         auto kern = field ? fwd_tc_fused<true> : fwd_tc_fused<false>;
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-            cudaSuccess)
+        if (!allow_smem(kern, smem))
           e = fail(NK_ERR_CUDA, "fwd_tc_fused: shared memory attribute");
         else {
           kern<<<(unsigned)B->start[B->n], Fwd<1>::THREADS, smem, st>>>(*B);
@@ -1255,13 +1253,11 @@ nk_status launch_adj_tc(const AdjTcArgs& A, const void* sigma_t, cudaStream_t st
   const size_t smem = 1024 + 2 * (32768 + (size_t)A.na64 * 128) + 64;
   dim3 grid(tiles, A.splits);
   if (A.cplx) {
-    if (cudaFuncSetAttribute(adj_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem) != cudaSuccess)
+    if (!allow_smem(adj_tc_kernel<true>, smem))
       return fail(NK_ERR_CUDA, "adj_tc: shared memory attribute");
     adj_tc_kernel<true><<<grid, kAdjThreads, smem, st>>>(map, A, chunk);
   } else {
-    if (cudaFuncSetAttribute(adj_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem) != cudaSuccess)
+    if (!allow_smem(adj_tc_kernel<false>, smem))
       return fail(NK_ERR_CUDA, "adj_tc: shared memory attribute");
     adj_tc_kernel<false><<<grid, kAdjThreads, smem, st>>>(map, A, chunk);
   }
@@ -1363,8 +1359,7 @@ static unsigned vec_blocks(int64_t elems) {
 nk_status launch_fwd_tc_batch(const FwdBatch& P, int G, int max_tiles, int max_na64,
                               cudaStream_t st) {
   const size_t smem = fwd_smem_bytes<0>(max_na64, kFwdBatchStages);
-  if (cudaFuncSetAttribute(fwd_tc_batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem) != cudaSuccess)
+  if (!allow_smem(fwd_tc_batch, smem))
     return fail(NK_ERR_CUDA, "fwd_tc_batch: shared memory attribute");
   fwd_tc_batch<<<dim3((unsigned)max_tiles, 1, (unsigned)G), Fwd<0>::THREADS, smem, st>>>(P);
   return check_launch("fwd_tc_batch");
@@ -1373,8 +1368,7 @@ nk_status launch_fwd_tc_batch(const FwdBatch& P, int G, int max_tiles, int max_n
 nk_status launch_adj_tc_batch(const AdjBatch& P, int G, int max_tiles, int max_splits,
                               int max_na64, cudaStream_t st) {
   const size_t smem = 1024 + 2 * (32768 + (size_t)max_na64 * 128) + 64;
-  if (cudaFuncSetAttribute(adj_tc_batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem) != cudaSuccess)
+  if (!allow_smem(adj_tc_batch, smem))
     return fail(NK_ERR_CUDA, "adj_tc_batch: shared memory attribute");
   adj_tc_batch<<<dim3((unsigned)max_tiles, (unsigned)max_splits, (unsigned)G), kAdjThreads, smem,
                  st>>>(P);
