@@ -1170,15 +1170,25 @@ constexpr int kCgCtas = 8;       // portable cluster size
 constexpr int kCgPer = 4;        // elements per thread of the vector updates
 constexpr int kCgMaxM = 63;      // one group of four columns per lane covers m + 1
 
-// The rule: one block's vectors, one column group, and so few samples and products that
-// eight SMs keep up with the whole GPU.  50 iterations, three launches each -> here, ms:
-// real 10 sites x 10 units, 1008 samples 1.81 -> 0.94, 4096 samples 1.66 -> 1.44; 20 x 40,
-// 1200 samples 2.87 -> 2.37; beyond the line, 20 x 20, 2000 samples 2.29 -> 2.37; complex
-// 14 x 14, 1500 samples 2.38 -> 1.74; beyond, 3000 samples 2.30 -> 3.06.
-static bool cg_small(int64_t ns, int m, int64_t pa, int cplx) {
-  const int64_t work = ns * pa;
-  return pa <= kCgPer * kVecThreads && m <= kCgMaxM && ns <= 4096 &&
-         work <= (ns <= 1536 ? 1 << 20 : cplx ? 1 << 18 : 1 << 19);
+// Where it is taken: problems that it has room for, and of those the ones whose busiest
+// CTA has so little to do, in tiles of 64 samples (forward) and rounds of 256 products
+// per sample of a split (adjoint), that it is done before three launches are; these take
+// longer with more hidden units.  50 iterations here and in three launches, ms: real
+// 10 x 10, 1200 samples 1.32 and 1.80, 20 x 20, 1200 samples 1.58 and 2.01, beyond the line
+// 1500 samples 2.08 and 2.01; complex 14 x 14, 1500 samples 1.82 and 2.01, beyond 2000
+// samples 2.12 and 2.05; 20 x 40, 600 samples 1.83 and 2.68, beyond 1200 samples 2.82 and
+// 2.64.  (Complex problems of more than 1536 samples and 2^18 products win or lose within
+// 6 % whatever the line.  Of 206 shapes measured, on the wrong side by more than that:
+// real 8 x 8, 3000 samples, 7 %.)
+static bool cg_small(int64_t ns, int m, int64_t pa, int cplx, int splits) {
+  if (pa > kCgPer * kVecThreads || m > kCgMaxM || ns > 4096) return false;
+  const int tiles = ceil_div(ceil_div((int)ns, 64), kCgCtas);
+  const int rounds = ceil_div(ceil_div((int)pa, kCgCtas) * splits, kVecThreads);
+  const int64_t adjoint = rounds * adjoint_chunk(ns, splits);
+  const int64_t cols = pa / (m + 1) * ceil_div(m + 1, 16);  // of a tile's products, per lane
+  if (cplx && ns > 1536 && ns * pa > 1 << 18) return false;
+  return cplx ? tiles * (100 + 2 * cols) + adjoint <= 750 + 8 * m
+              : tiles * 100 + adjoint <= 840 + 2 * m;
 }
 
 template <bool CPLX>
@@ -1186,7 +1196,7 @@ struct CgSmallSmem {
   using DT = typename D<CPLX>::T;
   using F = typename std::conditional<CPLX, float2, float>::type;
   DT p[kCgPer * kVecThreads];
-  F xf[kCgPer * kVecThreads];   // p as F32
+  F xf[kCgPer * kVecThreads + kCgMaxM + 1];  // p as F32, rows a pitch apart
   DT part[64][17];              // a tile's row sums by lane
   DT y[64];
   DT sh8[8];
@@ -1221,16 +1231,22 @@ __global__ void __cluster_dims__(kCgCtas, 1, 1) __launch_bounds__(kVecThreads)
   const int nvb = (ns + 63) / 64, vb0 = nvb * c / kCgCtas, vb1 = nvb * (c + 1) / kCgCtas;
   const int e0 = pa * c / kCgCtas, ec = pa * (c + 1) / kCgCtas - e0;
   const double invn = 1.0 / (double)ns;
+  // pitch of xf: lanes read neighbouring rows, which fall into the same banks where the
+  // pitch is a multiple of 16 (complex, 16 rows of 8 bytes: even); complex 15 x 30, 1500
+  // samples 2.95 -> 2.16 ms
+  const int xp = (na & (CPLX ? 1 : 15)) ? na : na + 1;
+  int at[kCgPer];  // where the thread's elements lie in it
   DT x[kCgPer], r[kCgPer];
 #pragma unroll
   for (int u = 0; u < kCgPer; ++u) {
     const int e = tid + u * kVecThreads;
     x[u] = r[u] = D<CPLX>::zero();
+    at[u] = xp == na ? e : e + e / na;
     if (e < pa) {
       r[u] = reinterpret_cast<const DT*>(A.r)[e];
       S.p[e] = r[u];
-      if constexpr (CPLX) S.xf[e] = make_float2((float)r[u].x, (float)r[u].y);
-      else S.xf[e] = (float)r[u];
+      if constexpr (CPLX) S.xf[at[u]] = make_float2((float)r[u].x, (float)r[u].y);
+      else S.xf[at[u]] = (float)r[u];
     }
   }
   double rs = A.scal[SC_RS0];
@@ -1247,7 +1263,7 @@ __global__ void __cluster_dims__(kCgCtas, 1, 1) __launch_bounds__(kVecThreads)
       const F* X[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        X[q] = S.xf + min(xl + 16 * q, m) * na;
+        X[q] = S.xf + min(xl + 16 * q, m) * xp;
 #pragma unroll
         for (int k = 0; k < 4; ++k) acc[q][k] = F{};
       }
@@ -1488,8 +1504,8 @@ __global__ void __cluster_dims__(kCgCtas, 1, 1) __launch_bounds__(kVecThreads)
         if (e >= pa) break;
         const DT pn = axpy(beta, S.p[e], r[u]);
         S.p[e] = pn;
-        if constexpr (CPLX) S.xf[e] = make_float2((float)pn.x, (float)pn.y);
-        else S.xf[e] = (float)pn;
+        if constexpr (CPLX) S.xf[at[u]] = make_float2((float)pn.x, (float)pn.y);
+        else S.xf[at[u]] = (float)pn;
       }
     }
     ++it;
@@ -1998,7 +2014,7 @@ static nk_status sr_step_t(nk_rbm* r, const int8_t* sigma, const void* T, const 
     fused_grid = std::max(fused_grid, std::min(ceil_div((int)L.pa, spread), kFusedPerSm * sms));
     if (ceil_div((int)L.pa, spread) > fused_grid) spread = 0;
   }
-  const bool small = !tc && !sy && cg_small(ns, m, L.pa, CPLX);
+  const bool small = !tc && !sy && cg_small(ns, m, L.pa, CPLX, splits);
   if (small && n_cg > 0) {
     const CgSmall A{sigma, T, weights, (int)ns, n, m, splits, (int)adjoint_chunk(ns, splits),
                     (int)L.pa, sc + L.x, sc + L.r, sc + L.y, sc + L.ap, red + 2 * kVecBlocks,
