@@ -1024,7 +1024,7 @@ __global__ void __launch_bounds__(256, 2) local_energy_wide(const __grid_constan
 }
 
 // Clusters of `parts` CTAs of a wide kernel that run at once (less than the SMs would
-// give, where a GPC's do not divide by the cluster).
+// give, where a GPC's do not divide by the cluster); 0 where none do.
 template <class K>
 static int64_t wide_slots(K kern, size_t smem, int parts) {
   cudaLaunchConfig_t cfg{};
@@ -1039,9 +1039,9 @@ static int64_t wide_slots(K kern, size_t smem, int parts) {
   cfg.numAttrs = 1;
   int n = 0;
   if (!allow_smem(kern, smem) ||
-      cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) {
+      cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
     cudaGetLastError();
-    return 1;
+    return 0;
   }
   return n;
 }
@@ -1095,7 +1095,7 @@ static WidePlan wide_plan(int64_t ns, int n_moves, bool cplx) {
                                     : wide_clusters<true, 2>(parts, alone))
                          : (np == 4 ? wide_clusters<false, 4>(parts, alone)
                                     : wide_clusters<false, 2>(parts, alone));
-        if (alone && tiles > at_once) continue;
+        if (at_once < 1 || (alone && tiles > at_once)) continue;
         const double cost = (double)((tiles + at_once - 1) / at_once) *
                             ((ntile + parts - 1) / parts) * (np == 4 ? 1.0 : cplx ? 0.6 : 0.75) *
                             (alone ? 1.0 : cplx ? 1.8 : 1.4);

@@ -2052,10 +2052,15 @@ static nk_status sr_step_t(nk_rbm* r, const int8_t* sigma, const void* T, const 
       CgFused A{sc + L.part, splits, L.pa, corner, sc + L.x, sc + L.r, sc + L.p, sc + L.ap, eps,
                 rtol,        red,    scal, it,     nbp,    spread, po};
       void* args[] = {&A};
-      if (cudaLaunchCooperativeKernel(cg_fused_kernel<CPLX>, dim3((unsigned)fused_grid), dim3(kVecThreads),
-                                      args, 0, st) != cudaSuccess)
-        return fail(NK_ERR_CUDA, "nk_sr_step: cooperative launch failed");
-      continue;
+      const cudaError_t e = cudaLaunchCooperativeKernel(
+          cg_fused_kernel<CPLX>, dim3((unsigned)fused_grid), dim3(kVecThreads), args, 0, st);
+      if (e == cudaSuccess) continue;
+      if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorNotSupported)
+        return fail(NK_ERR_CUDA, "nk_sr_step: cooperative launch failed: %s", cudaGetErrorString(e));
+      // refused, as in a context with fewer SMs than the device: three launches from here
+      // on, which make the same sums
+      cudaGetLastError();
+      fused_grid = 0;
     }
     if (sy) {  // S_t p_t + eps p_t = P^T (S P p_t) + eps p_t
       reduce_parts_kernel<CPLX><<<nbp, kVecThreads, 0, st>>>(
