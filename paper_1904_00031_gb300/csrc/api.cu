@@ -876,6 +876,16 @@ nk_status nk_tune_shapes(nk_rbm* rbm, const void* op_dev, int32_t n_moves, const
       return fail(NK_ERR_SHAPE, "nk_tune_shapes: scratch of %zu B, need %zu B (256-B aligned)",
                   scratch_bytes, need);
     r.theta_segs = rbm->theta_segs;
+    // real RBMs and site-quad operators run the same split for either count, which only
+    // orders a product's chunks: they keep the built-in one
+    OpDevHeader H;
+    if (cudaMemcpyAsync(&H, op_dev, sizeof(H), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaStreamSynchronize(st) != cudaSuccess)
+      return fail(NK_ERR_CUDA, "nk_tune_shapes: reading the operator failed");
+    if (!r.is_complex || (H.flags & kOpQuadMoves)) {
+      rbm->eloc_segs = local_energy_segs(n_moves, ns);
+      return NK_OK;
+    }
     float best = 1e30f;
     int best_s = 0;
     for (int segs = 1; segs <= 2; ++segs) {

@@ -78,6 +78,8 @@ nk_status launch_local_energy(const nk_rbm* r, const void* op_dev, int n_moves,
                               const int8_t* sigma, const void* theta, int64_t ns, double* eloc,
                               void* t_out, void* scratch, size_t scratch_bytes, cudaStream_t st);
 size_t local_energy_scratch_bytes(int m, int cplx, int n_moves);
+// nk_rbm.eloc_segs where it is 0
+int local_energy_segs(int n_moves, int64_t ns);
 // The local energies of items[idx[0..n)] fused into one move-table launch and one
 // energy launch per field (items already checked).
 nk_status launch_local_energy_fused(const nk_eloc_item* items, const int* idx, int n,

@@ -1143,6 +1143,17 @@ size_t local_energy_scratch_bytes(int m, int cplx, int n_moves) {
   return (size_t)(move_factor_offset(cplx, padded_m(m), (int)nm_pad) + nm_pad * 4 * 16);
 }
 
+// Two CTAs per SM: when the last wave of CTAs would be far from full, the move tiles of a
+// configuration tile are split into two halves (twice the CTAs) to even out the waves.
+int local_energy_segs(int n_moves, int64_t ns) {
+  const int64_t blocks = (ns + kEBS - 1) / kEBS;
+  auto wave_eff = [&](int64_t b) {
+    const int64_t slots = 2 * 152;
+    return (double)b / (double)(((b + slots - 1) / slots) * slots);
+  };
+  return (n_moves > kEBM && wave_eff(2 * blocks) > wave_eff(blocks)) ? 2 : 1;
+}
+
 // Everything one local-energy call needs, before anything is enqueued.
 struct ElocPlan {
   ElocArgs A;
@@ -1196,15 +1207,8 @@ static nk_status plan_local_energy(const nk_rbm* r, const void* op_dev, int n_mo
   P->smem = 2 * kEBK * kEBM * 16 + round_up(2 * kEBK * kETS * 16, 16) + 3 * kEBM * 4 +
             kEBM * 4 * 16 + 4 * 256 * 16 + 16;  // of local_energy_body
   P->blocks = (ns + kEBS - 1) / kEBS;
-  // two CTAs per SM: when the last wave of CTAs would be far from full, split
-  // the move tiles into two halves (twice the CTAs) to even out the waves
-  const int ntile = (n_moves + kEBM - 1) / kEBM;
-  auto wave_eff = [&](int64_t b) {
-    const int64_t slots = 2 * 152;
-    return (double)b / (double)(((b + slots - 1) / slots) * slots);
-  };
-  A.nseg = (ntile >= 2 && wave_eff(2 * P->blocks) > wave_eff(P->blocks)) ? 2 : 1;
-  if (r->eloc_segs > 0) A.nseg = (r->eloc_segs >= 2 && ntile >= 2) ? 2 : 1;  // tuned or set
+  A.nseg = local_energy_segs(n_moves, ns);
+  if (r->eloc_segs > 0) A.nseg = (r->eloc_segs >= 2 && n_moves > kEBM) ? 2 : 1;  // tuned or set
   A.seg_fast = A.nseg == 2 && P->blocks <= 65535 ? 1 : 0;
   P->wide = !cplx || (n_moves > 0 && n_moves % kEBM == 0);
   if (P->wide) P->wp = wide_plan(ns, n_moves, cplx);
