@@ -67,7 +67,7 @@ __device__ __forceinline__ typename FT<CPLX>::F tanh_t(typename FT<CPLX>::F h) {
 // Measured at [400, 1600, 400] complex, 16,384 samples, forward + backward: 18.2 ms
 // with scalar operands staged per 64 x 64 tile, 13.0 with packed instructions on
 // operands staged ready-made (192 bytes per 64 instructions: shared-memory bound,
-// FMA pipe 57 %), 10.2 as here (FMA pipe 68 %; 6.7 at the measured FMA rate).
+// FMA pipe 57 %), 10.0 as here (6.7 at the measured FMA rate).
 template <int MUL, int TR>
 struct GemmSmem {
   using L = Tile<MUL, TR>;
@@ -339,12 +339,14 @@ struct FfnnLayout {
   }
 };
 
-// Rows per thread of a contraction: 8 when its tiles (128 rows) fill every SM's
-// two CTAs and do not pad the rows much more than 64-row tiles would; else 4
-// (twice the CTAs, three to an SM).  Forward + backward of [400, 1600, 400] complex
-// on 16,384 samples: 10.3 ms with 8 everywhere, 10.4 with 4 everywhere.
-int tile_rows(int64_t rows, int64_t col_tiles, int z) {
+// Rows per thread of a contraction; forward + backward times.  Complex: 4 (64 rows, three
+// CTAs to an SM; [400, 1600, 400], 16,384 samples 10.0 ms, 128 rows 10.4; 4096 samples 2.72
+// and 3.32) as far as a grid's y goes.  Real: 8 when its tiles (128 rows) fill every SM's
+// two CTAs and do not pad the rows much more than 64-row tiles would (16,384 samples 4.45
+// ms, 64 rows everywhere 4.95; but [40, 160, 40] 355 us, 128 rows everywhere 389).
+int tile_rows(bool cplx, int64_t rows, int64_t col_tiles, int z) {
   const int64_t t8 = (rows + 127) / 128, t4 = (rows + 63) / 64;
+  if (cplx) return t4 > 65535 ? 8 : 4;
   return t8 * col_tiles * z >= 2 * 152 && 8 * t8 * 128 <= 9 * t4 * 64 ? 8 : 4;
 }
 
@@ -354,7 +356,7 @@ template <int MUL, class K8, class K4, class... Args>
 nk_status gemm_launch(K8 kern8, K4 kern4, int64_t rows, int64_t cols, int z, cudaStream_t st,
                       Args... args) {
   const int64_t ct = (cols + Tile<MUL, 8>::BC - 1) / Tile<MUL, 8>::BC;
-  const int tr = tile_rows(rows, ct, z);
+  const int tr = tile_rows(Tile<MUL, 4>::CPLX, rows, ct, z);
   const dim3 grid((unsigned)ct, (unsigned)((rows + 16 * tr - 1) / (16 * tr)), (unsigned)z);
   auto go = [&](auto kern, size_t smem) -> nk_status {
     if (smem > 48 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
