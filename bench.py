@@ -161,7 +161,7 @@ def run_oracle_all_cores(workload: str, n_chains: int, spc: int, n_cg: int,
 # single-pass ncu capture (dram__bytes_read.sum + dram__bytes_write.sum) of the
 # workload at full size; a kernel that changed since its capture has no entry.
 NCU_TRAFFIC = {
-    ("j1j2_20x20_alpha4", "bf16x2", "local_energy_tiled"): 9.327e9 + 0.864e9,
+    ("j1j2_20x20_alpha4", "bf16x2", "local_energy_wide"): 22.076e9 + 1.316e9,
 }
 
 ORACLE_SAMPLE = {"c5": (24, 2, 50), "c3": (64, 1, 50), "c2": (128, 4, 50), "c1": (16, 63, 120),
@@ -474,7 +474,12 @@ def run_gpu(args):
         rl[st_name] = {"bound": "tensor" if tensor else "alu", "achieved": round(ach, 3),
                        "peak": round(peak, 1), "unit": "TFLOP/s", "frac": round(ach / peak, 4)}
     dom = max(stage_ms, key=stage_ms.get)
-    kern = {"sample": "metropolis_kernel", "energies": "local_energy_tiled",
+    # real RBMs and complex ones on site-quad operators run the wide form (the flags of the
+    # compiled operator's header)
+    quads = bool(v.op.dev[28:32].view(torch.int32).item() & 1)
+    kern = {"sample": "metropolis_kernel",
+            "energies": ("local_energy_wide" if quads or not w.is_complex
+                         else "local_energy_tiled"),
             "amplitudes": ("fwd_tc_kernel (theta only)" if prec_name == "bf16x2"
                            else "logpsi_fp32_kernel (theta only)"),
             "sr": "SR step (fwd_tc + adj_tc + CG vector kernels)" if prec_name == "bf16x2"
