@@ -287,11 +287,11 @@ __device__ __forceinline__ void visible_term(const double* a, int n, const unsig
   for (int i = t; i < (CPLX ? 2 : 1) * n; i += 128)
     top = max(top, (uint32_t)__double2hiint(a[i]) & 0x7ff00000u);
   top = __reduce_max_sync(0xffffffffu, top);
-  uint32_t* tops = reinterpret_cast<uint32_t*>(tab);
+  uint32_t* tops = reinterpret_cast<uint32_t*>(tab + 448);
   if ((t & 31) == 0) tops[t >> 5] = top;
   asm volatile("bar.sync 2, 128;" ::: "memory");
+#pragma unroll
   for (int u = 0; u < 4; ++u) top = max(top, tops[u]);
-  asm volatile("bar.sync 2, 128;" ::: "memory");
   // f(i, -1 or 0) for 8 sites at a time, -1 where sigma_i < 0 (columns beyond n: 0)
   auto each_site = [&](auto&& f) {
 #pragma unroll 1
@@ -313,11 +313,15 @@ __device__ __forceinline__ void visible_term(const double* a, int n, const unsig
     return;
   }
   const int unit = max((int)(top >> 20), 1) - 1023 - 52;  // log2
+  // x 2^e (one multiplication where 2^e is a normal number)
+  auto times_pow2 = [](double x, int e) {
+    return e > -1000 && e < 1000 ? x * __longlong_as_double((long long)(1023 + e) << 52) : scalbn(x, e);
+  };
   for (int i = t; i < (int)round_up(n, 8); i += 128) {
     longlong2 v = make_longlong2(0, 0);
     if (i < n) {
-      v.x = __double2ll_rn(scalbn(a[CPLX ? 2 * i : i], -unit));
-      if (CPLX) v.y = __double2ll_rn(scalbn(a[2 * i + 1], -unit));
+      v.x = __double2ll_rn(times_pow2(a[CPLX ? 2 * i : i], -unit));
+      if (CPLX) v.y = __double2ll_rn(times_pow2(a[2 * i + 1], -unit));
     }
     tab[i] = v;
   }
@@ -330,8 +334,8 @@ __device__ __forceinline__ void visible_term(const double* a, int n, const unsig
     if (CPLX) hi += v.y ^ (long long)neg;
     negs -= neg;
   });
-  sr = scalbn((double)(hr + negs), unit);
-  if (CPLX) si = scalbn((double)(hi + negs), unit);
+  sr = times_pow2((double)(hr + negs), unit);
+  if (CPLX) si = times_pow2((double)(hi + negs), unit);
   asm volatile("bar.sync 2, 128;" ::: "memory");  // the table's tile goes back to staging
 }
 
