@@ -67,10 +67,24 @@ __device__ __forceinline__ typename FT<CPLX>::F tanh_t(typename FT<CPLX>::F h) {
 // Measured at [400, 1600, 400] complex, 16,384 samples, forward + backward: 18.2 ms
 // with scalar operands staged per 64 x 64 tile, 13.0 with packed instructions on
 // operands staged ready-made (192 bytes per 64 instructions: shared-memory bound,
-// FMA pipe 57 %), 10.0 as here (6.7 at the measured FMA rate).
+// FMA pipe 57 %), 9.6 as here (6.7 at the measured FMA rate).
+// The tiles of 16 TR rows.  Real ones of 64 rows have 64 columns (4 x 4 elements per
+// thread) in chunks of 16, two operand sets ahead: they run where CTAs are few, and a
+// CTA that has its SM to itself takes twice as long for twice the columns.
+template <int MUL, int TR>
+struct FTileOf {
+  using T = Tile<MUL, TR>;
+};
+template <>
+struct FTileOf<kMulReal, 4> {
+  using T = Tile<kMulReal, 4, false, 16, 64>;
+};
+template <int MUL, int TR>
+using FTile = typename FTileOf<MUL, TR>::T;
+
 template <int MUL, int TR>
 struct GemmSmem {
-  using L = Tile<MUL, TR>;
+  using L = FTile<MUL, TR>;
   static constexpr int PT = L::CPLX ? L::BC + 8 : L::BC + 16;  // row pitch of the result tile
   static constexpr size_t bytes() {
     const size_t tile = (size_t)L::BR * PT * (L::CPLX ? 8 : 4);
@@ -82,14 +96,14 @@ template <int MUL, int TR, class OA, class OB, class Epi>
 __device__ __forceinline__ void gemm_tile(int64_t R, int64_t C, int64_t kb, int64_t ke,
                                           int64_t r0, int64_t c0, OA& oa, OB& ob,
                                           const Epi& epi) {
-  using L = Tile<MUL, TR>;
+  using L = FTile<MUL, TR>;
   constexpr bool CPLX = L::CPLX;
   constexpr int PT = GemmSmem<MUL, TR>::PT;
   extern __shared__ __align__(16) unsigned char smraw[];
   L acc;
   acc.zero();
   acc.bounds(R - r0, C - c0);
-  acc.template run<1>(smraw, (int)((ke - kb + L::kFK - 1) / L::kFK), oa, ob, [](int) {});
+  acc.template run<L::kFK == 16 ? 2 : 1>(smraw, (int)((ke - kb + L::kFK - 1) / L::kFK), oa, ob, [](int) {});
   // The tile goes through shared memory so that the epilogue is a rolled loop (its
   // transcendentals, inlined once per element of the register tile, would not fit
   // the instruction cache) over whole row segments.
@@ -163,16 +177,16 @@ __global__ void __launch_bounds__(kFThreads, TR == 8 ? 2 : 3) ffnn_fwd_kernel(co
     if (H) H[s * wout + j] = h;
     Y[s * wout + j] = lncosh_t<CPLX>(h);
   };
-  const int64_t r0 = (int64_t)blockIdx.y * (16 * TR), c0 = (int64_t)blockIdx.x * Tile<MUL, TR>::BC;
-  using L = Tile<MUL, TR>;
-  Operand<F, false, L::BC, L::NB> ob;
+  using L = FTile<MUL, TR>;
+  const int64_t r0 = (int64_t)blockIdx.y * L::BR, c0 = (int64_t)blockIdx.x * L::BC;
+  Operand<F, false, L::BC, L::NB, false, false, false, false, L::kFK> ob;
   ob.init(Wm, win, c0, wout, 0, win);
   if constexpr (FIRST) {
-    Operand<int8_t, false, L::BR, L::NA> oa;
+    Operand<int8_t, false, L::BR, L::NA, false, false, false, false, L::kFK> oa;
     oa.init(sigma, win, r0, ns, 0, win);
     gemm_tile<MUL, TR>(ns, wout, 0, win, r0, c0, oa, ob, epi);
   } else {
-    Operand<F, false, L::BR, L::NA> oa;
+    Operand<F, false, L::BR, L::NA, false, false, false, false, L::kFK> oa;
     oa.init(X, win, r0, ns, 0, win);
     gemm_tile<MUL, TR>(ns, wout, 0, win, r0, c0, oa, ob, epi);
   }
@@ -226,10 +240,10 @@ __global__ void __launch_bounds__(kFThreads, TR == 8 ? 2 : 3) ffnn_bwd_kernel(co
     Eo[s * wprev + i] = cmul(cconj(tanh_t<CPLX>(H[s * wprev + i])), acc);
   };
   constexpr int MUL = CPLX ? kMulFull : kMulReal;
-  using L = Tile<MUL, TR>;
-  const int64_t r0 = (int64_t)blockIdx.y * (16 * TR), c0 = (int64_t)blockIdx.x * L::BC;
-  Operand<F, false, L::BR, L::NA> oa;
-  Operand<F, true, L::BC, L::NB, true> ob;
+  using L = FTile<MUL, TR>;
+  const int64_t r0 = (int64_t)blockIdx.y * L::BR, c0 = (int64_t)blockIdx.x * L::BC;
+  Operand<F, false, L::BR, L::NA, false, false, false, false, L::kFK> oa;
+  Operand<F, true, L::BC, L::NB, true, false, false, false, L::kFK> ob;
   oa.init(E, wl, r0, ns, 0, wl);
   ob.init(Wm, wprev, c0, wprev, 0, wl);
   gemm_tile<MUL, TR>(ns, wprev, 0, wl, r0, c0, oa, ob, epi);
@@ -250,16 +264,16 @@ __global__ void __launch_bounds__(kFThreads, TR == 8 ? 2 : 3) ffnn_wgrad_kernel(
   F* part = reinterpret_cast<F*>(partv) + (int64_t)blockIdx.z * wl * (wprev + 1);
   auto epi = [&](int64_t j, int64_t i, F acc) { part[j * (wprev + 1) + i] = acc; };
   const int64_t kb = (int64_t)blockIdx.z * chunk, ke = std::min<int64_t>(ns, kb + chunk);
-  const int64_t r0 = (int64_t)blockIdx.y * (16 * TR), c0 = (int64_t)blockIdx.x * Tile<MUL, TR>::BC;
-  using L = Tile<MUL, TR>;
-  Operand<F, true, L::BR, L::NA> oa;
+  using L = FTile<MUL, TR>;
+  const int64_t r0 = (int64_t)blockIdx.y * L::BR, c0 = (int64_t)blockIdx.x * L::BC;
+  Operand<F, true, L::BR, L::NA, false, false, false, false, L::kFK> oa;
   oa.init(E, wl, r0, wl, kb, ke);
   if constexpr (FIRST) {
-    Operand<int8_t, true, L::BC, L::NB, false, true> ob;
+    Operand<int8_t, true, L::BC, L::NB, false, true, false, false, L::kFK> ob;
     ob.init(sigma, wprev, c0, wprev + 1, kb, ke);
     gemm_tile<MUL, TR>(wl, wprev + 1, kb, ke, r0, c0, oa, ob, epi);
   } else {
-    Operand<F, true, L::BC, L::NB, true, true> ob;
+    Operand<F, true, L::BC, L::NB, true, true, false, false, L::kFK> ob;
     ob.init(X, wprev, c0, wprev + 1, kb, ke);
     gemm_tile<MUL, TR>(wl, wprev + 1, kb, ke, r0, c0, oa, ob, epi);
   }
@@ -339,33 +353,39 @@ struct FfnnLayout {
   }
 };
 
-// Rows per thread of a contraction; forward + backward times.  Complex: 4 (64 rows, three
-// CTAs to an SM; [400, 1600, 400], 16,384 samples 10.0 ms, 128 rows 10.4; 4096 samples 2.72
-// and 3.32) as far as a grid's y goes.  Real: 8 when its tiles (128 rows) fill every SM's
-// two CTAs and do not pad the rows much more than 64-row tiles would (16,384 samples 4.45
-// ms, 64 rows everywhere 4.95; but [40, 160, 40] 355 us, 128 rows everywhere 389).
-int tile_rows(bool cplx, int64_t rows, int64_t col_tiles, int z) {
-  const int64_t t8 = (rows + 127) / 128, t4 = (rows + 63) / 64;
-  if (cplx) return t4 > 65535 ? 8 : 4;
-  return t8 * col_tiles * z >= 2 * 152 && 8 * t8 * 128 <= 9 * t4 * 64 ? 8 : 4;
+// Rows per thread of a contraction: 8 (128 rows) where its tiles fill every SM's two CTAs
+// and do not pad the rows much more than 64-row tiles would, else 4.  Real, forward +
+// backward: [400, 1600, 400], 16,384 samples 4.45 ms, 64 x 128 tiles everywhere 4.95; on
+// 64 x 64 tiles [400, 800, 800, 400], 500 samples 355 us, 64 x 128 792.  Complex with the
+// sample operand real (a first layer's forward): [400, 800], 16,384 samples 585 us, 64
+// rows 691.  The other complex contractions keep 64 rows, three CTAs to an SM, as far as a
+// grid's y goes: [400, 400, 400, 400], 6000 samples, backward 1526 us, 128 rows where they
+// fill 1764; [400, 800], 16,384 samples, backward 1074 and 1218.
+template <int MUL>
+int tile_rows(int64_t rows, int64_t cols, int z) {
+  constexpr int BC = FTile<MUL, 8>::BC;
+  const int64_t t8 = (rows + 127) / 128, t4 = (rows + 63) / 64, ct = (cols + BC - 1) / BC;
+  if (MUL == kMulFull || MUL == kMulRealB) return t4 > 65535 ? 8 : 4;
+  return t8 * ct * z >= 2 * 152 && 8 * t8 * 128 <= 9 * t4 * 64 ? 8 : 4;
 }
 
-// Launches kern8 or kern4 (the two tile heights of one contraction) over
-// rows x cols x z.
+// Launches kern8 or kern4 (the two tiles of one contraction) over rows x cols x z.
 template <int MUL, class K8, class K4, class... Args>
 nk_status gemm_launch(K8 kern8, K4 kern4, int64_t rows, int64_t cols, int z, cudaStream_t st,
                       Args... args) {
-  const int64_t ct = (cols + Tile<MUL, 8>::BC - 1) / Tile<MUL, 8>::BC;
-  const int tr = tile_rows(Tile<MUL, 4>::CPLX, rows, ct, z);
-  const dim3 grid((unsigned)ct, (unsigned)((rows + 16 * tr - 1) / (16 * tr)), (unsigned)z);
-  auto go = [&](auto kern, size_t smem) -> nk_status {
+  using L8 = FTile<MUL, 8>;
+  using L4 = FTile<MUL, 4>;
+  auto go = [&](auto kern, int br, int bc, size_t smem) -> nk_status {
+    const dim3 grid((unsigned)((cols + bc - 1) / bc), (unsigned)((rows + br - 1) / br), (unsigned)z);
     if (smem > 48 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  (int)smem) != cudaSuccess)
       return fail(NK_ERR_CUDA, "nk_ffnn: shared memory attribute");
     kern<<<grid, kFThreads, smem, st>>>(args...);
     return NK_OK;
   };
-  return tr == 8 ? go(kern8, GemmSmem<MUL, 8>::bytes()) : go(kern4, GemmSmem<MUL, 4>::bytes());
+  return tile_rows<MUL>(rows, cols, z) == 8
+             ? go(kern8, L8::BR, L8::BC, GemmSmem<MUL, 8>::bytes())
+             : go(kern4, L4::BR, L4::BC, GemmSmem<MUL, 4>::bytes());
 }
 
 // The forward through all layers.  keep_h: h_l is stored for the backward, and
