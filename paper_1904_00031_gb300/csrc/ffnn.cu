@@ -62,12 +62,6 @@ __device__ __forceinline__ typename FT<CPLX>::F tanh_t(typename FT<CPLX>::F h) {
   }
 }
 
-// C[r][c] = sum_{k in [kb, ke)} A(r, k) B(c, k) for one tile (fgemm.cuh); epi(r, c,
-// acc) receives every element of the tile that lies inside R x C.
-// Measured at [400, 1600, 400] complex, 16,384 samples, forward + backward: 18.2 ms
-// with scalar operands staged per 64 x 64 tile, 13.0 with packed instructions on
-// operands staged ready-made (192 bytes per 64 instructions: shared-memory bound,
-// FMA pipe 57 %), 9.6 as here (6.7 at the measured FMA rate).
 // The tiles of 16 TR rows.  Real ones of 64 rows have 64 columns (4 x 4 elements per
 // thread) in chunks of 16, two operand sets ahead: they run where CTAs are few, and a
 // CTA that has its SM to itself takes twice as long for twice the columns.
@@ -82,6 +76,12 @@ struct FTileOf<kMulReal, 4> {
 template <int MUL, int TR>
 using FTile = typename FTileOf<MUL, TR>::T;
 
+// C[r][c] = sum_{k in [kb, ke)} A(r, k) B(c, k) for one tile (fgemm.cuh); epi(r, c,
+// acc) receives every element of the tile that lies inside R x C.
+// Measured at [400, 1600, 400] complex, 16,384 samples, forward + backward: 18.2 ms
+// with scalar operands staged per 64 x 64 tile, 13.0 with packed instructions on
+// operands staged ready-made (192 bytes per 64 instructions: shared-memory bound,
+// FMA pipe 57 %), 9.6 as here (6.7 at the measured FMA rate).
 template <int MUL, int TR>
 struct GemmSmem {
   using L = FTile<MUL, TR>;

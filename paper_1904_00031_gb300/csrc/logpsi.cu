@@ -28,6 +28,7 @@ struct LogpsiArgs {
   double* logpsi;     // c128 [ns], or null: theta / tanh(theta) only, no ln cosh
   F* theta_out;       // [ns][m] or null
   F* t_out;           // [ns][m] tanh(theta) or null
+  int segs;           // CTAs per sample tile, each with its share of the hidden tiles
 };
 
 // s + e += x exactly (Knuth's TwoSum in FP32, two values at a time)
@@ -40,27 +41,38 @@ __device__ __forceinline__ void two_sum2(float2& s, float2& e, float2 x) {
   s = t;
 }
 
-// One CTA: 64 samples, all hidden units in tiles of 64.
+// CTAs per sample tile of a call of `tiles`: theta and tanh(theta) are independent by
+// hidden tile, which are dealt out while CTAs are fewer than two per SM (complex 100 x
+// 400, 300 samples: 125 us with one, 23 here; 50 x 100, 8192 samples 26.8 and 19.8).
+static int logpsi_segs(const double* logpsi, int m, int64_t tiles) {
+  return logpsi ? 1 : (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(m, 64), 2 * 152 / tiles));
+}
+
+// One CTA: 64 samples, all hidden units (or the segment's) in tiles of 64.
 // Every 16-site chunk is summed in a fresh accumulator and carried with TwoSum, so
 // that theta is accurate to about one FP32 rounding instead of growing with the
 // number of sites; the units of a row are folded four at a time (x + 16 q of a tile)
 // in FP32, then in FP64.  At 10x10 real (16,383 samples, m = 400) theta
 // takes 79 us (scalar 4 x 4 blocks: 118; 128-unit tiles, whose sums did not fit the
 // registers: 118).
-template <bool CPLX>
+// (SEGS = false: one CTA per sample tile; as a run-time count it cost complex calls 3 %.)
+template <bool CPLX, bool SEGS>
 __device__ __forceinline__ void logpsi_fp32_body(const LogpsiArgs<CPLX>& A, int bx) {
   using F = typename LogpsiArgs<CPLX>::F;
   using L = Tile<CPLX ? kMulRealA : kMulReal, kLpTR, true, 16, 64>;
   __shared__ __align__(16) unsigned char smem[L::STAGE_BYTES];
-  const int64_t s0 = (int64_t)bx * kLpBS;
+  const int segs = SEGS ? A.segs : 1;
+  const int64_t s0 = (int64_t)(bx / segs) * kLpBS;
   const int n = A.n, m = A.m, K = n + 1;
+  const int jt = (m + L::BC - 1) / L::BC, seg = bx % segs;  // hidden tiles, this CTA's share
+  const int jt0 = jt * seg / segs, jt1 = jt * (seg + 1) / segs;
   __shared__ double2 psum[kLpTR][kFThreads];  // each thread's own sums, out of registers
 #pragma unroll
   for (int p = 0; p < kLpTR; ++p) psum[p][threadIdx.x] = make_double2(0.0, 0.0);
   Operand<int8_t, false, L::BR, L::NA, false, false, true, false, 16> oa;
   Operand<F, false, L::BC, L::NB, false, false, false, true, 16> ob;
   oa.init(A.sigma, n, s0, A.ns, 0, K);
-  ob.init(A.xw, K, 0, m, 0, K);
+  ob.init(A.xw, K, jt0 * L::BC, m, 0, K);
   L acc;
   float2 sx[L::TP][L::TC], ex[L::TP][L::TC];
   float2 sy[CPLX ? L::TP : 1][L::TC], ey[CPLX ? L::TP : 1][L::TC];
@@ -78,8 +90,8 @@ __device__ __forceinline__ void logpsi_fp32_body(const LogpsiArgs<CPLX>& A, int 
   acc.zero();
   acc.bounds(A.ns - s0, m);
   const int nk = (K + 15) / 16;  // chunks per tile of hidden units
-  int kc = 0, j0 = 0;
-  acc.template run<1>(smem, nk * ((m + L::BC - 1) / L::BC), oa, ob, [&](int) {
+  int kc = 0, j0 = jt0 * L::BC;
+  acc.template run<1>(smem, nk * (jt1 - jt0), oa, ob, [&](int) {
 #pragma unroll
     for (int p = 0; p < L::TP; ++p)
 #pragma unroll
@@ -158,9 +170,9 @@ __device__ __forceinline__ void logpsi_fp32_body(const LogpsiArgs<CPLX>& A, int 
   }
 }
 
-template <bool CPLX>
+template <bool CPLX, bool SEGS>
 __global__ void __launch_bounds__(kFThreads, 2) logpsi_fp32_kernel(LogpsiArgs<CPLX> A) {
-  logpsi_fp32_body<CPLX>(A, blockIdx.x);
+  logpsi_fp32_body<CPLX, SEGS>(A, blockIdx.x);
 }
 
 // Up to kLogpsiBatch problems of one field in one launch: CTA b runs sample
@@ -173,42 +185,51 @@ struct LogpsiFp32Batch {
   LogpsiArgs<CPLX> j[kLogpsiBatch];
 };
 
-template <bool CPLX>
+template <bool CPLX, bool SEGS>
 __global__ void __launch_bounds__(kFThreads, 2)
     logpsi_fp32_batch(const __grid_constant__ LogpsiFp32Batch<CPLX> B) {
   int k = 0;
   while (k + 1 < B.n && (int)blockIdx.x >= B.start[k + 1]) ++k;
-  logpsi_fp32_body<CPLX>(B.j[k], (int)blockIdx.x - B.start[k]);
+  logpsi_fp32_body<CPLX, SEGS>(B.j[k], (int)blockIdx.x - B.start[k]);
 }
 
 template <bool CPLX>
 static LogpsiArgs<CPLX> logpsi_args(const nk_rbm* r, const int8_t* sigma, int64_t ns,
-                                    double* logpsi, void* theta_out, void* t_out) {
+                                    double* logpsi, void* theta_out, void* t_out, int segs) {
   using F = typename LogpsiArgs<CPLX>::F;
   WsLayout L(r->n, r->m, r->is_complex);
   return LogpsiArgs<CPLX>{sigma, ns, r->n, r->m, (const F*)((const char*)r->ws + L.xw), r->a,
-                          logpsi, (F*)theta_out, (F*)t_out};
+                          logpsi, (F*)theta_out, (F*)t_out, segs};
 }
 
 // the problems of one field, at most kLogpsiBatch to a launch
 template <bool CPLX>
 static nk_status logpsi_fp32_field(const nk_logpsi_item* items, const int* idx, int n,
                                    cudaStream_t st) {
+  int64_t tiles = 0;
+  for (int u = 0; u < n; ++u)
+    if ((items[idx[u]].rbm->is_complex != 0) == CPLX)
+      tiles += (items[idx[u]].ns + kLpBS - 1) / kLpBS;
   for (int u0 = 0; u0 < n;) {
     LogpsiFp32Batch<CPLX> B;
     B.n = 0;
     B.start[0] = 0;
+    bool split = false;
     int u = u0;
     for (; u < n && B.n < kLogpsiBatch; ++u) {
       const nk_logpsi_item& it = items[idx[u]];
       if ((it.rbm->is_complex != 0) != CPLX) continue;
-      B.j[B.n] = logpsi_args<CPLX>(it.rbm, it.sigma, it.ns, it.logpsi_out, it.theta_out, nullptr);
-      B.start[B.n + 1] = B.start[B.n] + (int)((it.ns + kLpBS - 1) / kLpBS);
+      const int64_t t = (it.ns + kLpBS - 1) / kLpBS;
+      const int segs = logpsi_segs(it.logpsi_out, it.rbm->m, tiles);
+      split = split || segs > 1;
+      B.j[B.n] = logpsi_args<CPLX>(it.rbm, it.sigma, it.ns, it.logpsi_out, it.theta_out, nullptr, segs);
+      B.start[B.n + 1] = B.start[B.n] + (int)(t * segs);
       ++B.n;
     }
     u0 = u;
     if (B.n == 0) continue;
-    logpsi_fp32_batch<CPLX><<<B.start[B.n], kFThreads, 0, st>>>(B);
+    auto kern = split ? logpsi_fp32_batch<CPLX, true> : logpsi_fp32_batch<CPLX, false>;
+    kern<<<B.start[B.n], kFThreads, 0, st>>>(B);
     if (nk_status e = check_launch("nk_batch_logpsi")) return e;
   }
   return NK_OK;
@@ -222,13 +243,16 @@ nk_status launch_logpsi_fp32_fused(const nk_logpsi_item* items, const int* idx, 
 
 nk_status launch_logpsi_fp32(const nk_rbm* r, const int8_t* sigma, int64_t ns, double* logpsi,
                              void* theta_out, cudaStream_t st, void* t_out) {
-  const unsigned blocks = (unsigned)((ns + kLpBS - 1) / kLpBS);
-  if (r->is_complex)
-    logpsi_fp32_kernel<true><<<blocks, kFThreads, 0, st>>>(
-        logpsi_args<true>(r, sigma, ns, logpsi, theta_out, t_out));
-  else
-    logpsi_fp32_kernel<false><<<blocks, kFThreads, 0, st>>>(
-        logpsi_args<false>(r, sigma, ns, logpsi, theta_out, t_out));
+  const int64_t tiles = (ns + kLpBS - 1) / kLpBS;
+  const int segs = logpsi_segs(logpsi, r->m, tiles);
+  const unsigned blocks = (unsigned)(tiles * segs);
+  if (r->is_complex) {
+    auto kern = segs > 1 ? logpsi_fp32_kernel<true, true> : logpsi_fp32_kernel<true, false>;
+    kern<<<blocks, kFThreads, 0, st>>>(logpsi_args<true>(r, sigma, ns, logpsi, theta_out, t_out, segs));
+  } else {
+    auto kern = segs > 1 ? logpsi_fp32_kernel<false, true> : logpsi_fp32_kernel<false, false>;
+    kern<<<blocks, kFThreads, 0, st>>>(logpsi_args<false>(r, sigma, ns, logpsi, theta_out, t_out, segs));
+  }
   return check_launch("nk_rbm_logpsi");
 }
 
