@@ -2009,7 +2009,13 @@ static nk_status sr_step_t(nk_rbm* r, const int8_t* sigma, const void* T, const 
   if (!sy && cudaGetDevice(&dev) == cudaSuccess)
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   int spread = 0, fused_grid = std::min(nbp, kFusedPerSm * sms);
-  if (nbp < sms / 2 && splits > 4) {  // few blocks: the smallest slices that stay under two per SM
+  // Few blocks with little to reduce gain less from the fusion than the grid barriers take
+  // (20 iterations, BF16 hi + lo, fused and in three launches: complex 100 x 100, 300
+  // samples 888 us and 807, 100 x 400, 600 samples 1138 and 1079, but 16 x 64, 1000 samples
+  // 650 and 691, 40 x 80, 1200 samples 746 and 860).
+  if (tc && nbp < sms / 2 && splits <= 8 + nbp / 8) {
+    fused_grid = 0;
+  } else if (nbp < sms / 2 && splits > 4) {  // the smallest slices that stay under two per SM
     for (spread = 32; spread < 256 && ceil_div((int)L.pa, spread) > 2 * sms; spread *= 2) {}
     fused_grid = std::max(fused_grid, std::min(ceil_div((int)L.pa, spread), kFusedPerSm * sms));
     if (ceil_div((int)L.pa, spread) > fused_grid) spread = 0;
