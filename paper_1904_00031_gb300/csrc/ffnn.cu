@@ -249,20 +249,40 @@ __global__ void __launch_bounds__(kFThreads, TR == 8 ? 2 : 3) ffnn_bwd_kernel(co
   gemm_tile<MUL, TR>(ns, wprev, 0, wl, r0, c0, oa, ob, epi);
 }
 
+// Where this layer's gradient (W then b, flat) holds element (j, i); i = wprev: b_j.
+__device__ __forceinline__ int64_t grad_index(int64_t j, int64_t i, int wl, int wprev) {
+  return i < wprev ? j * wprev + i : (int64_t)wl * wprev + j;
+}
+
 // partial[z][j][i] = sum_{s in split z} e_l[s][j] conj(x'_(l-1)[s][i]),
-// x' = [x | 1] (i = wprev is the bias column); layer 1 reads sigma
+// x' = [x | 1] (i = wprev is the bias column); layer 1 reads sigma.  Given grad (one
+// split), the gradient itself, as the reduction would write it: small calls are bound by
+// their launches.
 template <bool CPLX, bool FIRST, int TR>
 __global__ void __launch_bounds__(kFThreads, TR == 8 ? 2 : 3) ffnn_wgrad_kernel(const void* __restrict__ ein,
                                                                   const int8_t* __restrict__ sigma,
                                                                   const void* __restrict__ xprev,
                                                                   int64_t ns, int wl, int wprev,
-                                                                  int64_t chunk, void* partv) {
+                                                                  int64_t chunk, void* partv,
+                                                                  double* grad) {
   using F = typename FT<CPLX>::F;
   constexpr int MUL = CPLX ? (FIRST ? kMulRealB : kMulFull) : kMulReal;
   const F* E = reinterpret_cast<const F*>(ein);
   const F* X = reinterpret_cast<const F*>(xprev);
   F* part = reinterpret_cast<F*>(partv) + (int64_t)blockIdx.z * wl * (wprev + 1);
-  auto epi = [&](int64_t j, int64_t i, F acc) { part[j * (wprev + 1) + i] = acc; };
+  auto epi = [&](int64_t j, int64_t i, F acc) {
+    if (!grad) {
+      part[j * (wprev + 1) + i] = acc;
+      return;
+    }
+    const int64_t k = grad_index(j, i, wl, wprev);
+    if constexpr (CPLX) {
+      grad[2 * k] = 0.0 + (double)acc.x;
+      grad[2 * k + 1] = 0.0 + (double)acc.y;
+    } else {
+      grad[k] = 0.0 + (double)acc;
+    }
+  };
   const int64_t kb = (int64_t)blockIdx.z * chunk, ke = std::min<int64_t>(ns, kb + chunk);
   using L = FTile<MUL, TR>;
   const int64_t r0 = (int64_t)blockIdx.y * L::BR, c0 = (int64_t)blockIdx.x * L::BC;
@@ -299,7 +319,7 @@ __global__ void ffnn_wreduce_kernel(const void* __restrict__ partv, int splits, 
       }
     }
     const int64_t j = x / (wprev + 1), i = x % (wprev + 1);
-    const int64_t k = i < wprev ? j * wprev + i : (int64_t)wl * wprev + j;
+    const int64_t k = grad_index(j, i, wl, wprev);
     if constexpr (CPLX) {
       grad[2 * k] = r;
       grad[2 * k + 1] = im;
@@ -435,21 +455,24 @@ nk_status backward_t(const nk_ffnn* f, const FfnnLayout& Lo, const int8_t* sigma
   for (int l = Lo.L; l >= 1; --l) {
     const float* Wm = p32 + fs * Lo.off[l - 1];
     const int wl = Lo.w[l], wp = Lo.w[l - 1];
+    double* gl = grad + fs * Lo.off[l - 1];
+    double* direct = Lo.splits == 1 ? gl : nullptr;
     nk_status e;
     if (l == 1)
       e = gemm_launch<CPLX ? kMulRealB : kMulReal>(
           ffnn_wgrad_kernel<CPLX, true, 8>, ffnn_wgrad_kernel<CPLX, true, 4>, wl, wp + 1, Lo.splits,
           st, (const void*)ecur, sigma, (const void*)nullptr, ns, wl, wp, Lo.chunk,
-          (void*)(sc + Lo.part));
+          (void*)(sc + Lo.part), direct);
     else
       e = gemm_launch<CPLX ? kMulFull : kMulReal>(
           ffnn_wgrad_kernel<CPLX, false, 8>, ffnn_wgrad_kernel<CPLX, false, 4>, wl, wp + 1,
           Lo.splits, st, (const void*)ecur, sigma, (const void*)(sc + Lo.x[l - 2]), ns, wl, wp,
-          Lo.chunk, (void*)(sc + Lo.part));
+          Lo.chunk, (void*)(sc + Lo.part), direct);
     if (e) return e;
     const int64_t per = (int64_t)wl * (wp + 1);
-    ffnn_wreduce_kernel<CPLX><<<(unsigned)std::min<int64_t>(1024, (per + 255) / 256), 256, 0, st>>>(
-        sc + Lo.part, Lo.splits, wl, wp, grad + fs * Lo.off[l - 1]);
+    if (!direct)
+      ffnn_wreduce_kernel<CPLX><<<(unsigned)std::min<int64_t>(1024, (per + 255) / 256), 256, 0, st>>>(
+          sc + Lo.part, Lo.splits, wl, wp, gl);
     if (l > 1) {
       e = gemm_launch<CPLX ? kMulFull : kMulReal>(
           ffnn_bwd_kernel<CPLX, 8>, ffnn_bwd_kernel<CPLX, 4>, ns, wp, 1, st, (const void*)ecur,
