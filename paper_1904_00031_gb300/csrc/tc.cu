@@ -292,30 +292,22 @@ __device__ __forceinline__ void visible_term(const double* a, int n, const unsig
   asm volatile("bar.sync 2, 128;" ::: "memory");
 #pragma unroll
   for (int u = 0; u < 4; ++u) top = max(top, tops[u]);
-  // f(i, -1 or 0) for 8 sites at a time, -1 where sigma_i < 0 (columns beyond n: 0)
-  auto each_site = [&](auto&& f) {
-#pragma unroll 1
-    for (int i0 = 0; i0 < n; i0 += 8) {
-      const uint4 g = *reinterpret_cast<const uint4*>(sA + (size_t)(i0 >> 6) * 16384 +
-                                                      sw128_offset(row, i0 & 63));
-      const uint32_t pk[4] = {g.x, g.y, g.z, g.w};
-#pragma unroll
-      for (int e = 0; e < 8; ++e)
-        f(i0 + e, (int)(e & 1 ? pk[e >> 1] : pk[e >> 1] << 16) >> 31);
-    }
-  };
   if (top == 0x7ff00000u) {
-    each_site([&](int i, int neg) {
-      if (i >= n) return;
-      sr += neg ? -a[CPLX ? 2 * i : i] : a[CPLX ? 2 * i : i];
-      if (CPLX) si += neg ? -a[2 * i + 1] : a[2 * i + 1];
-    });
+#pragma unroll 1
+    for (int i = 0; i < n; ++i) {
+      const int8_t* p = reinterpret_cast<const int8_t*>(sA) + (size_t)(i >> 6) * 16384 +
+                        sw128_offset(row, i & 63);
+      const double sg = p[1] < 0 ? -1.0 : 1.0;  // the sign of a BF16
+      sr += sg * a[CPLX ? 2 * i : i];
+      if (CPLX) si += sg * a[2 * i + 1];
+    }
     return;
   }
   const int unit = max((int)(top >> 20), 1) - 1023 - 52;  // log2
-  // x 2^e (one multiplication where 2^e is a normal number)
+  // x 2^e, |e| < 1200, in two steps of normal numbers
   auto times_pow2 = [](double x, int e) {
-    return e > -1000 && e < 1000 ? x * __longlong_as_double((long long)(1023 + e) << 52) : scalbn(x, e);
+    auto pow2 = [](int k) { return __longlong_as_double((long long)(1023 + k) << 52); };
+    return x * pow2(e / 2) * pow2(e - e / 2);
   };
   for (int i = t; i < (int)round_up(n, 8); i += 128) {
     longlong2 v = make_longlong2(0, 0);
@@ -328,12 +320,20 @@ __device__ __forceinline__ void visible_term(const double* a, int n, const unsig
   asm volatile("bar.sync 2, 128;" ::: "memory");
   long long hr = 0, hi = 0;
   int negs = 0;  // -x = ~x + 1: the ones are counted
-  each_site([&](int i, int neg) {
-    const longlong2 v = tab[i];
-    hr += v.x ^ (long long)neg;
-    if (CPLX) hi += v.y ^ (long long)neg;
-    negs -= neg;
-  });
+#pragma unroll 1
+  for (int i0 = 0; i0 < n; i0 += 8) {  // (columns beyond n: positive or zero)
+    const uint4 g = *reinterpret_cast<const uint4*>(sA + (size_t)(i0 >> 6) * 16384 +
+                                                    sw128_offset(row, i0 & 63));
+    const uint32_t pk[4] = {g.x, g.y, g.z, g.w};
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int neg = (int)(e & 1 ? pk[e >> 1] : pk[e >> 1] << 16) >> 31;  // 0 or -1
+      const longlong2 v = tab[i0 + e];
+      hr += v.x ^ (long long)neg;
+      if (CPLX) hi += v.y ^ (long long)neg;
+      negs -= neg;
+    }
+  }
   sr = times_pow2((double)(hr + negs), unit);
   if (CPLX) si = times_pow2((double)(hi + negs), unit);
   asm volatile("bar.sync 2, 128;" ::: "memory");  // the table's tile goes back to staging
