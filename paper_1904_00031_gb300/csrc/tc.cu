@@ -278,7 +278,8 @@ __device__ __forceinline__ uint32_t sig_bits(const int8_t* sigma, int64_t s, int
 // 2^53 each, whose sum is exact.  Each a_i is rounded by at most half a unit, which a
 // running FP64 sum of the same terms does about as often.  An infinite or NaN a_i has
 // no such unit: FP64 adds then.  (Pairs of floats, 48 bits and FP32's range, took longer:
-// ln psi + gradient at 20x20, 65,536 samples 2.78 -> 2.76 ms.)
+// ln psi + gradient at 20x20, 65,536 samples 2.78 -> 2.75 ms; a supervised step of 10 sites,
+// bound by latency, 89.3 -> 89.7 us.)
 template <bool CPLX>
 __device__ __forceinline__ void visible_term(const double* a, int n, const unsigned char* sA,
                                              int row, longlong2* tab, double& sr, double& si) {
